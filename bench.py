@@ -243,6 +243,8 @@ def stage_kernels(flags):
         return "k_detect_sweeps", "k_detect_sweeps"
     if "oneloop" in flags:                # every iteration walks the cells again
         sweep = "k_oneloop"
+    elif "flow" in flags:                 # one launch holds every sweep
+        sweep = "k_flow"
     else:
         sweep = "k_pja_fused" if "fused" in flags else ("k_pja_lean" if "lean" in flags else "k_pja")
     contacts = "k_pairs_half+k_pairs_finish" if "half" in flags else "k_contacts"
@@ -277,7 +279,7 @@ def profile_traffic(kernel: str, workload: str, kernel_digest: str):
 def kernel_digest() -> str:
     import hashlib
     h = hashlib.sha256()
-    for name in ("gg_kernels.cu", "gg_device.cuh"):
+    for name in ("gg_kernels.cu", "gg_flow.cu", "gg_sweep.cuh", "gg_device.cuh"):
         with open(os.path.join(ROOT, "paper_2306_01369_gb300", "csrc", name), "rb") as f:
             h.update(f.read())
     return h.hexdigest()[:16]
@@ -774,7 +776,7 @@ def measure(sim, sc, steps, stream, torch, flush, workload="column", readback=No
     if sweep_kernel == contact_kernels:   # detection and sweeps in one launch per step
         roofs = [roof(sweep_kernel, pja_ms + con_ms, pja_b + con_b, len(sampled)), None]
     else:
-        sweep_launches = len(sampled) * (1 if sweep_kernel == "k_pja_fused" else sc.params.pja_iters)
+        sweep_launches = len(sampled) * (1 if sweep_kernel in ("k_pja_fused", "k_flow") else sc.params.pja_iters)
         roofs = [roof(sweep_kernel, pja_ms, pja_b, sweep_launches),
                  roof(contact_kernels, con_ms, con_b, len(sampled))]
         roofs.sort(key=lambda r: -r["share_of_step"])

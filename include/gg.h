@@ -428,6 +428,10 @@ GG_API uint32_t gg_tuning_selected(const gg_sim *sim);
                                together with the counts */
 #define GG_TUNE_ONELOOP 128u /* OneLoop (Sec. II-D): each iteration re-walks the neighbour cells
                                 and computes the responses there, not from stored records */
+#define GG_TUNE_FLOW 256u    /* all sweeps in one launch ordered by data: the contact records stay in
+                                shared memory, partners exchange tagged velocity estimates, no
+                                barrier (with more than 8 free bodies, free bodies in a batch, or pja_weight = 1 the
+                                set runs the split launches) */
 
 GG_API uint32_t gg_tuning_flags(uint32_t k);
 

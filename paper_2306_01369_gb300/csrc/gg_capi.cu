@@ -41,12 +41,13 @@ constexpr gg::LaunchShape shape(int pja_block, uint32_t bits, int fused_block = 
   s.serp = (bits & GG_TUNE_SERP) ? 1u : 0u;
   s.pre = (bits & GG_TUNE_PRELOAD) ? 1u : 0u;
   s.one = (bits & GG_TUNE_ONELOOP) ? 1u : 0u;
+  s.flow = (bits & GG_TUNE_FLOW) ? 1u : 0u;
   return s;
 }
 
 // Launch-shape sets accepted by gg_params.tuning (index k-1).
 constexpr uint32_t kL = GG_TUNE_LISTS, kLean = GG_TUNE_LEAN, kHalf = GG_TUNE_HALF, kDet = GG_TUNE_DETECT,
-                   kSerp = GG_TUNE_SERP, kPre = GG_TUNE_PRELOAD, kOne = GG_TUNE_ONELOOP;
+                   kSerp = GG_TUNE_SERP, kPre = GG_TUNE_PRELOAD, kOne = GG_TUNE_ONELOOP, kFlow = GG_TUNE_FLOW;
 const gg::LaunchShape kShapes[] = {
     shape(256, 0),  shape(128, 0), shape(512, 0), shape(64, 0),       // 1-4: sort, per-launch sweeps
     shape(256, 0, 1024), shape(256, 0, 512),                           // 5-6: all sweeps in one launch
@@ -57,7 +58,8 @@ const gg::LaunchShape kShapes[] = {
     shape(128, kSerp | kPre), shape(128, kL | kSerp | kPre), shape(128, kL | kHalf | kSerp | kPre),  // 16-18
     shape(128, kOne), shape(128, kL | kOne),                           // 19-20: OneLoop
     shape(128, kL | kHalf),                                            // 21
-    shape(128, kL | kLean | kHalf | kSerp)};                           // 22
+    shape(128, kL | kLean | kHalf | kSerp),                            // 22
+    shape(128, kFlow), shape(128, kL | kFlow), shape(128, kL | kHalf | kFlow)};  // 23-25: dataflow sweeps
 constexpr uint32_t kNumShapes = sizeof(kShapes) / sizeof(kShapes[0]);
 
 // n_h factors the autotuner tries when gg_params.hash_tune is set (the paper's 2n first)
@@ -66,6 +68,9 @@ constexpr uint32_t kNumHashFactors = sizeof(kHashFactors) / sizeof(kHashFactors[
 // cell edges (x r_max of each environment) it then tries when the cell size is not fixed
 constexpr double kCellFactors[] = {2.002, 2.2, 2.5};
 constexpr uint32_t kNumCellFactors = sizeof(kCellFactors) / sizeof(kCellFactors[0]);
+
+// Spheres the dataflow sweeps of a batch take at a time (see gg_flow.cu).
+constexpr uint32_t kWaveParticles = 300000;
 
 constexpr uint32_t kStateMagic = 0x31534747u;  // "GGS1"
 
@@ -299,6 +304,12 @@ gg_status set_shape(gg_sim *s, uint32_t k) {
     const int per = ls.detect ? gg::detect_sweeps_blocks_per_sm(ls.lists != 0, s->K)
                               : gg::fused_pja_blocks_per_sm(ls.fused_block);
     ls.fused_grid = per > 0 ? (uint32_t)(per * nsm) : 0;
+  }
+  if (ls.flow) {
+    int nsm = 0;
+    GG_CUDA(s, cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, s->device));
+    const int per = gg::flow_setup(s->F != 0, &ls.flow_pool);
+    ls.flow_grid = per > 0 ? (uint32_t)(per * nsm) : 0;
   }
   s->ls = ls;
   s->a.lists = ls.lists;
@@ -562,7 +573,7 @@ uint32_t gg_tuning_flags(uint32_t k) {
   const gg::LaunchShape &ls = kShapes[k - 1];
   return (ls.lists ? GG_TUNE_LISTS : 0u) | (ls.fused_block ? GG_TUNE_FUSED : 0u) | (ls.lean ? GG_TUNE_LEAN : 0u) |
          (ls.half ? GG_TUNE_HALF : 0u) | (ls.detect ? GG_TUNE_DETECT : 0u) | (ls.serp ? GG_TUNE_SERP : 0u) |
-         (ls.pre ? GG_TUNE_PRELOAD : 0u) | (ls.one ? GG_TUNE_ONELOOP : 0u);
+         (ls.pre ? GG_TUNE_PRELOAD : 0u) | (ls.one ? GG_TUNE_ONELOOP : 0u) | (ls.flow ? GG_TUNE_FLOW : 0u);
 }
 
 uint32_t gg_kernels_per_step(const gg_sim *sim) { return sim ? gg::kernels_per_step(sim->a, sim->ls) : 0; }
@@ -773,6 +784,29 @@ gg_status gg_create_batch(const gg_params *params, uint32_t n_envs, const uint32
   if ((rc = dalloc(s, &a.head, s->nh_cap)) || (rc = dalloc(s, &a.next, n)) || (rc = dalloc(s, &a.pcnt, n)) ||
       (rc = dalloc(s, &a.pscr, (size_t)2 * s->K * n)))
     return bail(rc);
+  // dataflow sweeps: tagged estimates, record scratch, and the particle ranges they take one
+  // after another (whole environments, as many as fit the shared memory of the chip)
+  uint32_t *wave_off = nullptr;
+  if ((rc = dalloc(s, &a.T[0], n)) || (rc = dalloc(s, &a.T[1], n)) ||
+      (rc = dalloc(s, &a.epoch, 1)) || (rc = dalloc(s, &a.farr, s->F)) || (rc = dalloc(s, &a.ftw, (size_t)s->F * 4)) ||
+      (rc = dalloc(s, &wave_off, (size_t)n_envs + 1)))
+    return bail(rc);
+  a.tag_step = P.pja_iters + 2u;
+  std::vector<uint32_t> waves{0u};
+  for (uint32_t e2 = 0; e2 < n_envs; ++e2) {
+    if (s->envs[e2].off > waves.back() && s->envs[e2].off + s->envs[e2].n - waves.back() > kWaveParticles)
+      waves.push_back(s->envs[e2].off);
+  }
+  waves.push_back(n);
+  a.n_waves = (uint32_t)waves.size() - 1u;
+  int nsm = 0;
+  if ((cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, s->device)) != cudaSuccess || nsm < 1) nsm = 1;
+  a.flow_region = gg::kFlowRecords;
+  const size_t rec = (size_t)nsm * a.flow_region;
+  if ((rc = dalloc(s, &a.tile_work, ((size_t)n + 31) / 32 + 4)) || (rc = dalloc(s, &a.flow_n, rec)) ||
+      (rc = dalloc(s, &a.flow_l, rec)) || (rc = dalloc(s, &a.flow_r, rec)) || (rc = dalloc(s, &a.flow_b, rec)))
+    return bail(rc);
+  a.wave_off = wave_off;
   a.F = s->F;
   a.Lcap = s->Lcap;
   s->fgb.assign(s->F, 0xffffffffu);
@@ -788,6 +822,7 @@ gg_status gg_create_batch(const gg_params *params, uint32_t n_envs, const uint32
     GG_UP(a.vel_id, h_vel.data(), sizeof(float4) * n);
     GG_UP(a.env_of, h_env.data(), sizeof(uint32_t) * n);
   }
+  GG_UP(wave_off, waves.data(), sizeof(uint32_t) * waves.size());
   GG_UP(a.envs, s->envs.data(), sizeof(DevEnv) * n_envs);
   GG_UP(a.chunk_env, h_chunk_env.data(), sizeof(uint32_t) * h_chunk_env.size());
 #undef GG_UP
@@ -801,6 +836,11 @@ gg_status gg_create_batch(const gg_params *params, uint32_t n_envs, const uint32
       (e = cudaMemset(a.sid, 0, sizeof(uint32_t) * std::max(n, 1u))) != cudaSuccess ||
       (e = cudaMemset(a.key_id, 0, sizeof(uint32_t) * std::max(n, 1u))) != cudaSuccess ||
       (e = cudaMemset(a.ctrl, 0, sizeof(DevCtrl))) != cudaSuccess ||
+      (e = cudaMemset(a.epoch, 0, sizeof(uint32_t))) != cudaSuccess ||
+      (e = cudaMemset(a.tile_work, 0, sizeof(uint32_t) * (((size_t)n + 31) / 32 + 4))) != cudaSuccess ||
+      (e = cudaMemset(a.T[0], 0, sizeof(float4) * std::max(n, 1u))) != cudaSuccess ||
+      (e = cudaMemset(a.T[1], 0, sizeof(float4) * std::max(n, 1u))) != cudaSuccess ||
+      (e = cudaMemset(a.ftw, 0, sizeof(float4) * std::max(4 * s->F, 1u))) != cudaSuccess ||
       (e = cudaMemset(a.ncb, 0, sizeof(uint32_t) * nbt)) != cudaSuccess ||
       (e = cudaMemset(a.fgb, 0xff, sizeof(uint32_t) * std::max(s->F, 1u))) != cudaSuccess ||
       (e = cudaMemset(a.fcount, 0, sizeof(uint32_t) * std::max(s->F, 1u))) != cudaSuccess ||

@@ -31,6 +31,9 @@ constexpr uint32_t kFlagBucketBound = 64u; // a bucket held more than kMaxBucket
 // and the step reports an error instead of running for minutes.
 constexpr uint32_t kMaxBucket = 1024;
 
+// Tags of the dataflow sweeps (gg_flow.cu) start over past this one.
+constexpr uint32_t kTagLimit = 0x30000000u;
+
 constexpr uint32_t kListEnd = 0xffffffffu;  // end of a bucket's linked list
 constexpr int kMaxK = 32;   // particle-particle capacity limit
 constexpr int kMaxKb = 8;   // particle-body capacity limit
@@ -172,6 +175,22 @@ struct StepArgs {
   float *wpart;           // [n_chunks][maxb][6]
   float *wrench;          // [wrench_hist][n_envs * maxb][6]
   DevCtrl *ctrl;
+  // dataflow sweeps (gg_flow.cu)
+  uint32_t flow;          // the step's sweeps run there (the contact build then leaves clam and blam unset)
+  uint32_t flow_fin;      // buffer of U^I
+  uint32_t n_waves;       // particle ranges [wave_off[w], wave_off[w + 1]) swept one after another
+  const uint32_t *wave_off;
+  float4 *T[2];           // tagged velocity estimates: x, y, z, tag (launch epoch + iteration)
+  uint32_t *tile_work;    // [ceil(n / 32)] per 32 spheres: their contacts this step, the most of one << 16
+  uint32_t flow_region;   // record scratch of one block (entries of the arrays below): what does not fit on chip
+  float4 *flow_n;         // [blocks][flow_region] normal, bias
+  float4 *flow_l;         // impulse, effective mass
+  uint2 *flow_r;          // place and flags, partner
+  float4 *flow_b;         // body contacts: point velocity or lever arm
+  uint32_t *epoch;        // tag base of the next launch
+  uint32_t tag_step;      // tags a step takes
+  uint32_t *farr;         // [F] free-body contacts updated so far in this launch
+  float4 *ftw;            // [F][2][2] a free body's (v, tag), (w, -) by iteration parity
   // free rigid bodies
   uint32_t F, Lcap;       // free-body slots, contact-list capacity per free body
   uint32_t *ncb;          // [n_envs * maxb] contacts per body this step

@@ -40,7 +40,20 @@ struct LaunchShape {
   uint32_t serp;        // serpentine sweeps: every other per-launch sweep runs its blocks in reverse
   uint32_t pre;         // per-launch sweeps load the first round's records with the counts
   uint32_t one;         // OneLoop: every iteration re-walks the cells and computes the responses
+  uint32_t flow;        // all sweeps in one launch ordered by data (gg_flow.cu) ...
+  uint32_t flow_grid;   // ... of this many blocks (all resident)
+  uint32_t flow_pool;   // ... and this much dynamic shared memory each
 };
+// Free bodies the dataflow sweeps take: each holds a block (an SM) of its own for the
+// whole launch, so more than a few would cost more than the sweeps gain.
+constexpr uint32_t kFlowMaxFree = 8;
+inline bool uses_flow(const StepArgs &a, const LaunchShape &ls) {
+  return ls.flow && ls.flow_grid > a.F && a.n < (1u << 29) && a.n && !a.lit && a.F <= kFlowMaxFree && (!a.F || a.n_waves == 1) && a.n_waves <= 1024u;
+}
+constexpr uint32_t kFlowRecords = 10240;      // record scratch of one block, for what does not fit on chip
+constexpr uint32_t kFlowMaxWaves = 1024;     // particle ranges of one launch
+int flow_setup(bool free, uint32_t *pool);  // resident blocks per SM, shared memory per block
+cudaError_t enqueue_flow(const StepArgs &a, const LaunchShape &ls, cudaStream_t st);
 int fused_pja_blocks_per_sm(int block);
 int detect_sweeps_blocks_per_sm(bool lists, uint32_t K);
 

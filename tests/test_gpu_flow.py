@@ -1,0 +1,154 @@
+"""The dataflow sweeps (launch-shape sets with GG_TUNE_FLOW: every sweep in one launch, the
+contact records on chip, partners' estimates exchanged as tagged values) against the
+per-launch sweeps: bit-identical positions, velocities, wrenches and impulses at the sizes
+where tiles, blocks and ranges end, with free bodies, several particle ranges, records
+that do not fit on chip, lists cut by the contact capacity, and bounded waits."""
+import dataclasses
+import time
+
+import numpy as np
+import pytest
+
+from gpu_helpers import need_gpu
+from paper_2306_01369_gb300 import scenes as S
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def gg():
+    need_gpu()
+    from paper_2306_01369_gb300 import gg as g
+    return g
+
+
+def flow_sets(gg):
+    return [k for k in range(1, gg.load().gg_tuning_count() + 1) if "flow" in gg.tuning_flags(k)]
+
+
+def squeezed(n, seed=11, factor=0.95, shuffle=False, **params):
+    """A box of overlapping spheres (about three contacts each)."""
+    sc = S.settle_box(n=max(n, 64), seed=seed)
+    pr = sc.pos_r[:n].copy()
+    pr[:, :3] *= np.float32(factor)
+    if shuffle:
+        pr = pr[np.argsort(S.uniform(seed, n), kind="stable")]
+    return S.Scene("squeezed", np.ascontiguousarray(pr), np.zeros((n, 3), np.float32), S.sphere_mass(pr[:, 3]), sc.bodies,
+                   dataclasses.replace(sc.params, **params), 10)
+
+
+def outputs(gg, sc, tuning, steps, check=True, **kw):
+    sim = gg.Sim.from_scene(sc, tuning=tuning, wrench_history=steps, **kw)
+    sim.step(steps)
+    out = [sim.read(f, check=check) for f in ("POS", "VEL", "BODY_STATE", "BODY_WRENCH", "CONTACT_IMPULSE",
+                                              "BODY_CONTACT_IMPULSE")]
+    out.append(sim.read("CONTACTS", np.uint32, check=check))
+    flags = sim.stats()["status_flags"]
+    sim.close()
+    return out, flags
+
+
+def same(gg, sc, steps=3, ref=7, sets=None, **kw):
+    want, wf = outputs(gg, sc, ref, steps, **kw)
+    for k in sets or flow_sets(gg):
+        got, gf = outputs(gg, sc, k, steps, **kw)
+        assert gf == wf
+        for a, b in zip(got, want):
+            assert np.array_equal(a, b), (sc.name, k)
+
+
+@pytest.mark.parametrize("n", [1, 2, 31, 32, 33, 1000, 4096])
+def test_sizes_around_a_tile(gg, n):
+    same(gg, squeezed(n))
+
+
+@pytest.mark.parametrize("iters", [1, 2, 3])
+def test_few_iterations(gg, iters):
+    same(gg, squeezed(2000, pja_iters=iters))
+
+
+def test_ids_in_no_spatial_order(gg):
+    same(gg, squeezed(4000, shuffle=True))
+
+
+def test_free_and_moving_bodies(gg):
+    same(gg, S.excavation(n=6000, n_steps=20), steps=12, sets=[flow_sets(gg)[-1]])
+
+
+def test_more_free_bodies_than_the_launch_takes(gg):
+    """Nine free bodies: the set runs the split launches."""
+    sc = squeezed(600)
+    top = float(sc.pos_r[:, 2].max())
+    sc.bodies = sc.bodies + [S.Body(kind=S.BOX, shape=(0.004,) * 3, pos=(0.03 + 0.015 * k, 0.05, top + 0.006), is_free=1,
+                                    mass=0.01, inertia=(1e-6,) * 3) for k in range(7)]
+    sc.bodies += [S.Body(kind=S.BOX, shape=(0.004,) * 3, pos=(0.03, 0.08 + 0.02 * k, top + 0.006), is_free=1, mass=0.01,
+                         inertia=(1e-6,) * 3) for k in range(2)]
+    same(gg, sc, max_bodies=16)
+
+
+def test_several_particle_ranges(gg):
+    """A batch of more spheres than one range takes, its environments uneven."""
+    b = S.batched_beds(n_envs=14, n_steps=4, n_min=15000, n_max=40000)
+    assert b.n > 300000
+    for e in range(14):
+        a, z = int(b.env_offsets[e]), int(b.env_offsets[e + 1])
+        b.pos_r[a:z, 1:3] *= np.float32(0.97)
+    same(gg, b, steps=2, sets=[flow_sets(gg)[1]])
+
+
+def test_records_beyond_the_shared_memory(gg):
+    """A crowded cloud in random order: about ten partners a sphere, most of them other
+    blocks' (their records do not all fit on chip)."""
+    n = 90000
+    pr, vel = S.random_cloud(n, 5, box=0.135, vel_scale=0.05)
+    sc = S.Scene("cloud", pr, vel, S.sphere_mass(pr[:, 3]), [S.Body(kind=S.PLANE, pos=(0.0, 0.0, -0.01))],
+                 S.Params(dt=1e-5, max_contacts=32), 4)
+    same(gg, sc, steps=1, sets=[flow_sets(gg)[1]])
+
+
+def test_lists_cut_by_the_capacity(gg):
+    """One-sided lists (a sphere with more partners than its capacity): the plain sweeps
+    run, as bit-identical as before."""
+    sc = squeezed(3000, factor=0.9, max_contacts=2)
+    want, wf = outputs(gg, sc, 7, 1, check=False)
+    assert wf & 1
+    for k in flow_sets(gg):
+        if "half" in gg.tuning_flags(k):
+            continue      # (which partners a half-stencil pass loses depends on its atomics)
+        got, gf = outputs(gg, sc, k, 1, check=False)
+        assert gf == wf
+        for a, b in zip(got, want):
+            assert np.array_equal(a, b), k
+
+
+def test_waits_run_out_and_report(gg):
+    """A phantom participant (tags that nothing writes): every wait runs out within its
+    bound, the step reports it, and the context stays usable."""
+    sc = squeezed(3000)
+    k = flow_sets(gg)[0]
+    sim = gg.Sim(sc.pos_r, sc.vel, sc.mass, sc.params, tuning=k, barrier_test_phantoms=1, wait_limit_us=20000)
+    sim.set_bodies(sc.bodies)
+    t0 = time.perf_counter()
+    sim.step(1)
+    with pytest.raises(gg.GGError) as e:
+        sim.sync()
+    assert e.value.status == gg.ERR_DEVICE_TIMEOUT
+    assert time.perf_counter() - t0 < 5.0
+    sim.close()
+    same(gg, sc, steps=2, sets=[k])
+
+
+def test_going_back_to_a_checkpoint(gg):
+    """Steps taken again from a restored state (the same step indices) equal the first
+    time's: no value published then is taken for one of now."""
+    sc = squeezed(3000)
+    sim = gg.Sim.from_scene(sc, tuning=flow_sets(gg)[1])
+    sim.step(2)
+    blob = sim.state()
+    sim.step(3)
+    first = [sim.pos(), sim.vel()]
+    for _ in range(2):
+        sim.set_state(blob)
+        sim.step(3)
+        assert np.array_equal(first[0], sim.pos()) and np.array_equal(first[1], sim.vel())
+    sim.close()
