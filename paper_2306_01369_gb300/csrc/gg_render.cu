@@ -8,6 +8,12 @@
 // image does not depend on the order of the spheres.  Bodies are sphere traced per
 // pixel (FP32, fixed order) and merged.  The decisions (coverage, ray-sphere hit,
 // every tracing step) use the same operations in the same order as the oracle.
+//
+// An image is a chain of short kernels (2 to 30 us each as separate launches), so they are
+// chained with programmatic dependent launch and each does as little as it can: the spheres
+// are taken last id first (beds are laid down bottom up, so what a camera above sees comes
+// early) and a value goes to its pixel's atomic only if it beats what is already there; a
+// ray stops being traced where the spheres already block it.
 #include <cuda_runtime.h>
 
 #include "gg_device.cuh"
@@ -28,6 +34,7 @@ __device__ __forceinline__ float from_ordered(uint32_t k) {
 }
 
 __global__ void k_fill(uint32_t *img, uint32_t count, uint32_t v) {
+  pdl_enter();
   const uint32_t p = blockIdx.x * blockDim.x + threadIdx.x;
   if (p < count) img[p] = v;
 }
@@ -37,9 +44,10 @@ __device__ __forceinline__ float pixel_centre(float base, uint32_t u, float step
 }
 
 __global__ void k_splat_height(StepArgs a, uint32_t off, uint32_t n, RenderArgs c, uint32_t *img) {
+  pdl_enter();
   const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
-  const float4 p = a.pos_id[off + i];
+  const float4 p = a.pos_id[off + (n - 1u - i)];
   // conservative pixel range: |x - px| <= r with px = bx + (u + 1/2) sx
   const int u0 = max(0, (int)floorf((p.x - p.w - c.bx) / c.sx - 0.5f) - 1);
   const int u1 = min((int)c.W - 1, (int)ceilf((p.x + p.w - c.bx) / c.sx - 0.5f) + 1);
@@ -55,12 +63,14 @@ __global__ void k_splat_height(StepArgs a, uint32_t off, uint32_t n, RenderArgs 
       const float d2 = __fadd_rn(__fmul_rn(dx, dx), __fmul_rn(dy, dy));
       if (!(d2 <= r2)) continue;
       const float h = __fadd_rn(p.z, __fsqrt_rn(__fsub_rn(r2, d2)));
-      atomicMax(&img[(size_t)v * c.W + u], ordered(h));
+      uint32_t *px_at = &img[(size_t)v * c.W + u];
+      if (ordered(h) > __ldcg(px_at)) atomicMax(px_at, ordered(h));  // (a pixel only grows)
     }
   }
 }
 
 __global__ void k_finish_height(const uint32_t *img, uint32_t count, float empty, float *out) {
+  pdl_enter();
   const uint32_t p = blockIdx.x * blockDim.x + threadIdx.x;
   if (p < count) out[p] = img[p] ? from_ordered(img[p]) : empty;
 }
@@ -81,18 +91,22 @@ __device__ __forceinline__ float3 pixel_ray(const RenderArgs &c, uint32_t u, uin
   return make_float3(d[0], d[1], d[2]);
 }
 
-// The ray of every pixel, once per image (the splat tests many spheres against each).
-__global__ void k_make_rays(RenderArgs c) {
+// Every pixel's ray, once per image (the splat tests many spheres against each), and its
+// empty value.
+__global__ void k_begin_depth(RenderArgs c, uint32_t *img) {
+  pdl_enter();
   const uint32_t p = blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= c.W * c.H) return;
   const float3 d = pixel_ray(c, p % c.W, p / c.W);
   c.rays[p] = make_float4(d.x, d.y, d.z, 0.f);
+  img[p] = 0x7f800000u;
 }
 
 __global__ void k_splat_depth(StepArgs a, uint32_t off, uint32_t n, RenderArgs c, uint32_t *img) {
+  pdl_enter();
   const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
-  const float4 p = a.pos_id[off + i];
+  const float4 p = a.pos_id[off + (n - 1u - i)];
   const float oc0 = __fsub_rn(p.x, c.o[0]), oc1 = __fsub_rn(p.y, c.o[1]), oc2 = __fsub_rn(p.z, c.o[2]);
   const float rr = __fmul_rn(p.w, p.w);
   // conservative footprint from the centre in the camera frame (any rounding here
@@ -121,7 +135,8 @@ __global__ void k_splat_depth(StepArgs a, uint32_t off, uint32_t n, RenderArgs c
       if (!(disc >= 0.0f)) continue;
       const float t0 = __fsub_rn(b, __fsqrt_rn(disc));
       if (!(t0 >= c.near && t0 <= c.far)) continue;
-      atomicMin(&img[(size_t)v * c.W + u], __float_as_uint(t0));  // t0 > 0: bits order as floats
+      uint32_t *px_at = &img[(size_t)v * c.W + u];
+      if (__float_as_uint(t0) < __ldcg(px_at)) atomicMin(px_at, __float_as_uint(t0));  // t0 > 0: bits order as floats
     }
 }
 
@@ -144,6 +159,7 @@ __device__ __forceinline__ float march_sdf(const DevBody &b, float3 y, float eps
 }
 
 __global__ void k_trace_depth(StepArgs a, uint32_t gb0, uint32_t nb, RenderArgs c, const uint32_t *img, float *out) {
+  pdl_enter();
   const uint32_t p = blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= c.W * c.H) return;
   float best = __uint_as_float(img[p]);
@@ -151,6 +167,9 @@ __global__ void k_trace_depth(StepArgs a, uint32_t gb0, uint32_t nb, RenderArgs 
     const float4 d = c.rays[p];
     float t = c.near;
     for (uint32_t k = 0; k < c.steps; ++k) {
+      // a hit from here on would lie behind the nearest sphere (t only grows): 96 steps of a
+      // 36 x 36 image over a bed took 33.8 us, the few in front of it 5
+      if (t >= best) break;
       const float3 x = make_float3(__fadd_rn(c.o[0], __fmul_rn(t, d.x)), __fadd_rn(c.o[1], __fmul_rn(t, d.y)),
                                    __fadd_rn(c.o[2], __fmul_rn(t, d.z)));
       float fmin = __int_as_float(0x7f800000);
@@ -177,16 +196,23 @@ inline unsigned cdiv(uint32_t a, unsigned b) { return a ? (a + b - 1) / b : 1; }
 cudaError_t enqueue_render(const StepArgs &a, uint32_t env_off, uint32_t env_n, uint32_t gb0, uint32_t nb,
                            const RenderArgs &c, uint32_t *img, float *out, cudaStream_t st) {
   const uint32_t np = c.W * c.H;
+  cudaError_t e;
+  bool first = true;
+#define GG_CHAIN(kern, count, block, ...)                                                        \
+  do {                                                                                           \
+    if ((e = launch(!first, kern, dim3(cdiv(count, block)), block, 0, st, __VA_ARGS__)) != cudaSuccess) return e; \
+    first = false;                                                                               \
+  } while (0)
   if (c.kind == 0) {
-    k_fill<<<cdiv(np, 256), 256, 0, st>>>(img, np, 0u);
-    if (env_n) k_splat_height<<<cdiv(env_n, 128), 128, 0, st>>>(a, env_off, env_n, c, img);
-    k_finish_height<<<cdiv(np, 256), 256, 0, st>>>(img, np, c.empty, out);
+    GG_CHAIN(k_fill, np, 256, img, np, 0u);
+    if (env_n) GG_CHAIN(k_splat_height, env_n, 128, a, env_off, env_n, c, img);
+    GG_CHAIN(k_finish_height, np, 256, (const uint32_t *)img, np, c.empty, out);
   } else {
-    k_fill<<<cdiv(np, 256), 256, 0, st>>>(img, np, 0x7f800000u);
-    k_make_rays<<<cdiv(np, 128), 128, 0, st>>>(c);
-    if (env_n) k_splat_depth<<<cdiv(env_n, 128), 128, 0, st>>>(a, env_off, env_n, c, img);
-    k_trace_depth<<<cdiv(np, 128), 128, 0, st>>>(a, gb0, nb, c, img, out);
+    GG_CHAIN(k_begin_depth, np, 128, c, img);
+    if (env_n) GG_CHAIN(k_splat_depth, env_n, 128, a, env_off, env_n, c, img);
+    GG_CHAIN(k_trace_depth, np, 128, a, gb0, nb, c, (const uint32_t *)img, out);
   }
+#undef GG_CHAIN
   return cudaGetLastError();
 }
 
