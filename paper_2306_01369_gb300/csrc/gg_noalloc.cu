@@ -8,6 +8,10 @@
 // the sort needs (bucket histogram, scan block sums, unsorted slot list) lives in
 // the file-scope array g_noalloc_scratch below, which every GPU that loads this
 // library holds until the process exits.  Sizes are limited by that array.
+//
+// Six short kernels of a few us each, so launches and their gaps are most of the time: they
+// are chained with programmatic dependent launch, and the scan has no kernel of its own for
+// the block sums (each down-sweep block adds up the sums before its own).
 #include <cuda_runtime.h>
 
 #include <cstring>
@@ -15,6 +19,7 @@
 
 #include "../../include/gg.h"
 #include "gg_device.cuh"
+#include "gg_internal.h"
 
 namespace {
 
@@ -26,7 +31,6 @@ constexpr uint32_t kNABlocks = kNABuckets / kNATile;                      // sca
 constexpr uint32_t kNAWords = kNABuckets + kNABlocks + GG_NOALLOC_MAX_PARTICLES;
 
 static_assert(kNABuckets % kNATile == 0, "bucket capacity must be a whole number of scan tiles");
-static_assert(kNABlocks <= 1024, "block sums are scanned by one block");
 
 // Scratch shared by every call on a device: [histogram | block sums | unsorted slots].
 static __device__ __align__(256) uint32_t g_noalloc_scratch[kNAWords];
@@ -36,16 +40,20 @@ std::mutex g_mutex;
 uint32_t *g_scratch_ptr[kMaxDevices] = {};
 
 __global__ void na_clear(uint32_t *cnt, uint32_t words) {
+  gg::pdl_enter();
   for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < words; i += gridDim.x * blockDim.x) cnt[i] = 0u;
 }
 
-__global__ void na_key(const float4 *pos, uint32_t n, float inv_cell, uint32_t nh, uint32_t *key, uint32_t *cnt) {
+// (a particle's arrival number in its bucket goes to `order`: the scatter needs no atomics)
+__global__ void na_key(const float4 *pos, uint32_t n, float inv_cell, uint32_t nh, uint32_t *key, uint32_t *cnt,
+                       uint32_t *order) {
+  gg::pdl_enter();
   const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const float4 p = pos[i];
   const uint32_t k = gg::hash_cell(gg::cell_of(p.x, inv_cell), gg::cell_of(p.y, inv_cell), gg::cell_of(p.z, inv_cell), nh);
   key[i] = k;
-  atomicAdd(&cnt[k], 1u);
+  order[i] = atomicAdd(&cnt[k], 1u);
 }
 
 __device__ __forceinline__ uint32_t na_warp_scan(uint32_t v) {
@@ -80,51 +88,67 @@ __device__ __forceinline__ uint32_t na_block_scan(uint32_t v, uint32_t *total) {
 }
 
 __global__ void __launch_bounds__(kNAThreads) na_reduce(const uint32_t *cnt, uint32_t *bsum) {
-  const uint32_t base = blockIdx.x * kNATile + threadIdx.x * kNAItems;
+  gg::pdl_enter();
+  const uint4 *c4 = reinterpret_cast<const uint4 *>(cnt + blockIdx.x * kNATile);
   uint32_t s = 0;
 #pragma unroll
-  for (uint32_t k = 0; k < kNAItems; ++k) s += cnt[base + k];
+  for (uint32_t k = 0; k < kNAItems / 4; ++k) {  // (a sum: any order, so the loads are coalesced)
+    const uint4 v = c4[k * kNAThreads + threadIdx.x];
+    s += v.x + v.y + v.z + v.w;
+  }
   uint32_t total;
   (void)na_block_scan(s, &total);
   if (threadIdx.x == 0) bsum[blockIdx.x] = total;
 }
 
-__global__ void __launch_bounds__(1024) na_top(uint32_t *bsum, uint32_t nblk, uint32_t *start, uint32_t nh) {
-  const uint32_t v = threadIdx.x < nblk ? bsum[threadIdx.x] : 0u;
-  uint32_t total;
-  const uint32_t ex = na_block_scan(v, &total);
-  if (threadIdx.x < nblk) bsum[threadIdx.x] = ex;
-  if (threadIdx.x == 0) start[nh] = total;
-}
-
 __global__ void __launch_bounds__(kNAThreads) na_down(const uint32_t *cnt, const uint32_t *bsum, uint32_t *start,
                                                       uint32_t nh) {
+  gg::pdl_enter();
   const uint32_t base = blockIdx.x * kNATile + threadIdx.x * kNAItems;
+  uint32_t before = 0;  // counts of the tiles before this one
+  for (uint32_t t = threadIdx.x; t < blockIdx.x; t += kNAThreads) before += bsum[t];
+  const uint4 *c4 = reinterpret_cast<const uint4 *>(cnt + base);
   uint32_t v[kNAItems], s = 0;
 #pragma unroll
-  for (uint32_t k = 0; k < kNAItems; ++k) {
-    v[k] = cnt[base + k];
-    s += v[k];
+  for (uint32_t k = 0; k < kNAItems / 4; ++k) {
+    const uint4 q = c4[k];
+    v[4 * k] = q.x;
+    v[4 * k + 1] = q.y;
+    v[4 * k + 2] = q.z;
+    v[4 * k + 3] = q.w;
+    s += q.x + q.y + q.z + q.w;
   }
-  uint32_t total;
-  uint32_t run = bsum[blockIdx.x] + na_block_scan(s, &total);
+  uint32_t total, first;
+  (void)na_block_scan(before, &first);
+  uint32_t run = first + na_block_scan(s, &total);
+  if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) start[nh] = first + total;
+  // through shared memory (a word of padding per 32), so that the table is written line by line
+  __shared__ uint32_t tab[kNATile + kNATile / 32];
 #pragma unroll
   for (uint32_t k = 0; k < kNAItems; ++k) {
-    if (base + k < nh) start[base + k] = run;
+    const uint32_t at = threadIdx.x * kNAItems + k;
+    tab[at + at / 32] = run;
     run += v[k];
+  }
+  __syncthreads();
+#pragma unroll
+  for (uint32_t k = 0; k < kNAItems; ++k) {
+    const uint32_t at = k * kNAThreads + threadIdx.x, b = blockIdx.x * kNATile + at;
+    if (b < nh) start[b] = tab[at + at / 32];
   }
 }
 
-__global__ void na_scatter(const uint32_t *key, uint32_t n, const uint32_t *start, uint32_t *cnt, uint32_t *slots) {
+__global__ void na_scatter(const uint32_t *key, uint32_t n, const uint32_t *start, const uint32_t *order, uint32_t *slots) {
+  gg::pdl_enter();
   const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
-  const uint32_t k = key[i];
-  slots[start[k] + atomicSub(&cnt[k], 1u) - 1u] = i;
+  slots[start[key[i]] + order[i]] = i;
 }
 
 // ascending id inside each bucket; a bucket above GG_NOALLOC_MAX_OCCUPANCY keeps the
 // scatter's order (the rank would cost its occupancy per member)
 __global__ void na_rank(const uint32_t *key, uint32_t n, const uint32_t *start, const uint32_t *slots, uint32_t *perm) {
+  gg::pdl_enter();
   const uint32_t s = blockIdx.x * blockDim.x + threadIdx.x;
   if (s >= n) return;
   const uint32_t id = slots[s];
@@ -175,15 +199,18 @@ extern "C" gg_status gg_bin_sort_noalloc(const float *pos_radius, uint32_t n, fl
   const uint32_t hist_words = nblk * kNATile;  // whole tiles: the scan reads them all
   uint32_t *cnt = scratch, *bsum = scratch + kNABuckets, *slots = bsum + kNABlocks;
   const uint32_t gp = (n + 255) / 256;
-  na_clear<<<(hist_words + 1023) / 1024, 1024, 0, s>>>(cnt, hist_words);
-  if (n) na_key<<<gp, 256, 0, s>>>(reinterpret_cast<const float4 *>(pos_radius), n, inv_cell, n_h, keys, cnt);
-  na_reduce<<<nblk, kNAThreads, 0, s>>>(cnt, bsum);
-  na_top<<<1, 1024, 0, s>>>(bsum, nblk, cell_start, n_h);
-  na_down<<<nblk, kNAThreads, 0, s>>>(cnt, bsum, cell_start, n_h);
-  if (n) {
-    na_scatter<<<gp, 256, 0, s>>>(keys, n, cell_start, cnt, slots);
-    na_rank<<<gp, 256, 0, s>>>(keys, n, cell_start, slots, perm);
-  }
-  const cudaError_t e = cudaGetLastError();
+  const float4 *pos = reinterpret_cast<const float4 *>(pos_radius);
+  cudaError_t e = gg::launch(false, na_clear, dim3((hist_words + 1023) / 1024), 1024, 0, s, cnt, hist_words);
+  if (n && e == cudaSuccess) e = gg::launch(true, na_key, dim3(gp), 256, 0, s, pos, n, inv_cell, n_h, keys, cnt, perm);
+  if (e == cudaSuccess) e = gg::launch(true, na_reduce, dim3(nblk), kNAThreads, 0, s, (const uint32_t *)cnt, bsum);
+  if (e == cudaSuccess)
+    e = gg::launch(true, na_down, dim3(nblk), kNAThreads, 0, s, (const uint32_t *)cnt, (const uint32_t *)bsum, cell_start, n_h);
+  if (n && e == cudaSuccess)
+    e = gg::launch(true, na_scatter, dim3(gp), 256, 0, s, (const uint32_t *)keys, n, (const uint32_t *)cell_start,
+                   (const uint32_t *)perm, slots);
+  if (n && e == cudaSuccess)
+    e = gg::launch(true, na_rank, dim3(gp), 256, 0, s, (const uint32_t *)keys, n, (const uint32_t *)cell_start,
+                   (const uint32_t *)slots, perm);
+  if (e != cudaSuccess) (void)cudaGetLastError();
   return e == cudaSuccess ? GG_OK : GG_ERR_CUDA;
 }
