@@ -128,6 +128,10 @@ struct gg_sim {
     uint32_t *ccount = nullptr, *cj = nullptr, *bj = nullptr;
     float4 *cn = nullptr, *bn = nullptr, *bxc = nullptr;
     gg::AdjArgs d{};
+    // the reverse pass's graphs, one per slot and direction, kept between reverse passes of
+    // the same length and tool (capturing them took 2 of 12 ms for 20 steps)
+    std::vector<cudaGraphExec_t> fwd, adj;
+    uint32_t graph_steps = 0, graph_tool = 0xffffffffu;
     std::vector<void *> allocs;
   } ad;
   bool timing = false;
@@ -194,7 +198,17 @@ gg_status read_ctrl(gg_sim *s, DevCtrl *out, cudaStream_t st) {
   return GG_OK;
 }
 
+void free_reverse_graphs(gg_sim *s) {
+  for (auto *v : {&s->ad.fwd, &s->ad.adj}) {
+    for (cudaGraphExec_t g : *v)
+      if (g) cudaGraphExecDestroy(g);
+    v->clear();
+  }
+}
+
+// Every captured graph: they bake in the launch shape, the tables and the step arguments.
 void free_graph(gg_sim *s) {
+  free_reverse_graphs(s);
   for (int t = 0; t < 2; ++t) {
     if (s->exec[t]) cudaGraphExecDestroy(s->exec[t]);
     if (s->graph[t]) cudaGraphDestroy(s->graph[t]);
@@ -1377,6 +1391,7 @@ gg_status gg_tape_reserve(gg_sim *s, uint32_t n_steps, uint32_t K) {
   if (s->a.lit) return fail(s, GG_ERR_UNSUPPORTED, "differentiation with pja_weight = 1 is not supported");
   if (n_steps == 0 || K == 0) return fail(s, GG_ERR_INVALID_ARG, "gg_tape_reserve: n_steps and K must be > 0");
   GG_CUDA(s, cudaDeviceSynchronize());
+  free_reverse_graphs(s);
   for (void *p : s->ad.allocs) cudaFree(p);
   s->ad.allocs.clear();
   s->ad.taped = 0;
@@ -1488,17 +1503,19 @@ gg_status gg_backward(gg_sim *s, const float *dL_dpos, const float *dL_dvel, con
   // index from the step counter restored with the state), captured when first needed,
   // so that the host captures the next graph while the device runs the previous one.
   const uint32_t slots = s->ad.slots;
-  std::vector<cudaGraphExec_t> fwd(slots, nullptr), adj(slots, nullptr);
-  struct ExecGuard {  // the graphs are destroyed on every return below, after their launches
-    std::vector<cudaGraphExec_t> *v[2];
+  std::vector<cudaGraphExec_t> &fwd = s->ad.fwd, &adj = s->ad.adj;
+  if (fwd.size() != slots || s->ad.graph_steps != N || s->ad.graph_tool != s->ad.tool) {
+    GG_CUDA(s, cudaStreamSynchronize(st));  // (an earlier reverse pass may still run them)
+    free_reverse_graphs(s);
+    fwd.assign(slots, nullptr);
+    adj.assign(slots, nullptr);
+    s->ad.graph_steps = N;
+    s->ad.graph_tool = s->ad.tool;
+  }
+  struct Wait {  // every return below waits for the launches
     cudaStream_t st;
-    ~ExecGuard() {
-      cudaStreamSynchronize(st);
-      for (auto *x : v)
-        for (cudaGraphExec_t g : *x)
-          if (g) cudaGraphExecDestroy(g);
-    }
-  } guard{{&fwd, &adj}, st};
+    ~Wait() { cudaStreamSynchronize(st); }
+  } guard{st};
   const gg::DevCtrl *ctrl0 = reinterpret_cast<const gg::DevCtrl *>(
       s->ad.ckpt + (size_t)n * 32 + (size_t)s->n_envs * s->maxb * sizeof(DevBody));
   auto launch_slot = [&](bool reverse, uint32_t slot) -> gg_status {

@@ -1221,6 +1221,52 @@ __device__ __forceinline__ void advance_pose(float dt, float p[3], float q[4], c
   }
 }
 
+// Free-box corners: +lambda on the box, -lambda on the other body, added to thread 0's v in
+// the order (box, corner, other body).  The block looks at kWrenchBodyThreads of them at a
+// time and thread 0 adds the few that count (one thread reading all of them in turn took
+// 35 us of the excavation's step).
+constexpr int kWrenchBodyThreads = 256;
+
+__device__ __forceinline__ void add_corners(const StepArgs &a, uint32_t gb, uint32_t e, const float p[3], float v[6]) {
+  __shared__ float sm[kWrenchBodyThreads][6];
+  __shared__ uint32_t on[kWrenchBodyThreads / 32];
+  const float inv_dt = 1.0f / a.dt;
+  const uint32_t per = 8u * a.maxb;
+  for (uint32_t t0 = 0; t0 < a.maxb * per; t0 += kWrenchBodyThreads) {
+    const uint32_t t = t0 + threadIdx.x, ob = t / per;
+    float sg = 0.f;
+    if (t < a.maxb * per) {
+      const DevBody &Fb = a.bodies[e * a.maxb + ob];
+      if (Fb.active && Fb.is_free) {
+        const CornerContact &c = a.fcc[(size_t)Fb.fid * per + t % per];
+        if (c.valid) sg = (e * a.maxb + ob == gb) ? inv_dt : ((e * a.maxb + c.o == gb) ? -inv_dt : 0.f);
+        if (sg != 0.f) {
+          const float fx = sg * c.lam[0], fy = sg * c.lam[1], fz = sg * c.lam[2];
+          const float rx = c.xc[0] - p[0], ry = c.xc[1] - p[1], rz = c.xc[2] - p[2];
+          float *d = sm[threadIdx.x];
+          d[0] = fx;
+          d[1] = fy;
+          d[2] = fz;
+          d[3] = ry * fz - rz * fy;
+          d[4] = rz * fx - rx * fz;
+          d[5] = rx * fy - ry * fx;
+        }
+      }
+    }
+    const uint32_t m = __ballot_sync(0xffffffffu, sg != 0.f);
+    if ((threadIdx.x & 31u) == 0) on[threadIdx.x >> 5] = m;
+    if (!__syncthreads_or(sg != 0.f)) continue;
+    if (threadIdx.x == 0)
+      for (uint32_t w = 0; w < kWrenchBodyThreads / 32; ++w)
+        for (uint32_t mm = on[w]; mm; mm &= mm - 1u) {
+          const float *d = sm[32u * w + (uint32_t)__ffs((int)mm) - 1u];
+#pragma unroll
+          for (int q = 0; q < 6; ++q) v[q] += d[q];
+        }
+    __syncthreads();
+  }
+}
+
 // One block per body slot: sum its environment's chunk partials in a fixed order (a
 // thread per chunk, strided, then the block's fixed tree) into the wrench ring, then
 // advance the body's pose (no block reads another body's pose); a free body keeps the
@@ -1229,8 +1275,6 @@ __device__ __forceinline__ void advance_pose(float dt, float p[3], float q[4], c
 // chunks in turn was eight round trips deep on a 256-chunk environment: 10 us).  The
 // last block to finish advances the step counter (every block read it first; no block
 // waits for another).
-constexpr int kWrenchBodyThreads = 256;
-
 __global__ void __launch_bounds__(kWrenchBodyThreads) k_wrench_bodies(StepArgs a) {
   pdl_enter();
   const uint32_t gb = blockIdx.x;
@@ -1259,31 +1303,11 @@ __global__ void __launch_bounds__(kWrenchBodyThreads) k_wrench_bodies(StepArgs a
     }
   }
   block_sum6<kWrenchBodyThreads>(v);
+  if (active && a.F) add_corners(a, gb, e, p, v);
   if (threadIdx.x == 0) {
     if (gb == 0) {  // the tags of the next step's dataflow sweeps (0: k_key clears the old ones)
       const uint32_t e = *a.epoch + a.tag_step;
       *a.epoch = e > kTagLimit ? 0u : e;
-    }
-    if (active && a.F) {  // free-box corners: +lambda on the box, -lambda on the other body
-      const float inv_dt = 1.0f / a.dt;
-      for (uint32_t ob = 0; ob < a.maxb; ++ob) {
-        const DevBody &Fb = a.bodies[e * a.maxb + ob];
-        if (!Fb.active || !Fb.is_free) continue;
-        const CornerContact *cc = a.fcc + (size_t)Fb.fid * 8 * a.maxb;
-        for (uint32_t t = 0; t < 8 * a.maxb; ++t) {
-          if (!cc[t].valid) continue;
-          const float sg = (e * a.maxb + ob == gb) ? inv_dt : ((e * a.maxb + cc[t].o == gb) ? -inv_dt : 0.f);
-          if (sg == 0.f) continue;
-          const float fx = sg * cc[t].lam[0], fy = sg * cc[t].lam[1], fz = sg * cc[t].lam[2];
-          const float rx = cc[t].xc[0] - p[0], ry = cc[t].xc[1] - p[1], rz = cc[t].xc[2] - p[2];
-          v[0] += fx;
-          v[1] += fy;
-          v[2] += fz;
-          v[3] += ry * fz - rz * fy;
-          v[4] += rz * fx - rx * fz;
-          v[5] += rx * fy - ry * fx;
-        }
-      }
     }
     float *dst = a.wrench + ((size_t)(step % a.wrench_hist) * nbt + gb) * 6;
 #pragma unroll
