@@ -9,11 +9,14 @@
 // pixel (FP32, fixed order) and merged.  The decisions (coverage, ray-sphere hit,
 // every tracing step) use the same operations in the same order as the oracle.
 //
-// An image is a chain of short kernels (2 to 30 us each as separate launches), so they are
-// chained with programmatic dependent launch and each does as little as it can: the spheres
-// are taken last id first (beds are laid down bottom up, so what a camera above sees comes
-// early) and a value goes to its pixel's atomic only if it beats what is already there; a
-// ray stops being traced where the spheres already block it.
+// An image is a chain of short kernels, so they are chained with programmatic dependent
+// launch and each does as little as it can: the spheres are taken last id first (beds are
+// laid down bottom up, so what a camera above sees comes early) and a value goes to its
+// pixel's atomic only if it beats what is already there; a ray stops being traced where the
+// spheres already block it.  A 72 x 36 height map and a 36 x 36 depth image of 262,144
+// spheres: 60.7 -> 41.0 us, most of it k_depth.
+#include <algorithm>
+
 #include <cuda_runtime.h>
 
 #include "gg_device.cuh"
@@ -102,10 +105,26 @@ __global__ void k_begin_depth(RenderArgs c, uint32_t *img) {
   img[p] = 0x7f800000u;
 }
 
-__global__ void k_splat_depth(StepArgs a, uint32_t off, uint32_t n, RenderArgs c, uint32_t *img) {
-  pdl_enter();
-  const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
+// Distance used to step the tracing: the body's SDF; outside a GRID body's sampled box
+// the distance to that box, at least eps.
+__device__ __forceinline__ float march_sdf(const DevBody &b, float3 y, float eps) {
+  int br;
+  const float f = body_sdf(b, y, &br);
+  if (b.kind != 4 || br >= 0) return f;
+  const float yy[3] = {y.x, y.y, y.z};
+  float q[3];
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    const float lo = b.shape[k];
+    const float hi = __fadd_rn(b.shape[k], __fmul_rn(b.shape[3], (float)(b.gn[k] - 1u)));
+    q[k] = fmaxf(fmaxf(__fsub_rn(lo, yy[k]), __fsub_rn(yy[k], hi)), 0.0f);
+  }
+  const float s = __fadd_rn(__fadd_rn(__fmul_rn(q[0], q[0]), __fmul_rn(q[1], q[1])), __fmul_rn(q[2], q[2]));
+  return fmaxf(__fsqrt_rn(s), eps);
+}
+
+__device__ __forceinline__ void splat_depth(const StepArgs &a, uint32_t off, uint32_t n, const RenderArgs &c, uint32_t i,
+                                            uint32_t *img) {
   const float4 p = a.pos_id[off + (n - 1u - i)];
   const float oc0 = __fsub_rn(p.x, c.o[0]), oc1 = __fsub_rn(p.y, c.o[1]), oc2 = __fsub_rn(p.z, c.o[2]);
   const float rr = __fmul_rn(p.w, p.w);
@@ -140,53 +159,70 @@ __global__ void k_splat_depth(StepArgs a, uint32_t off, uint32_t n, RenderArgs c
     }
 }
 
-// Distance used to step the tracing: the body's SDF; outside a GRID body's sampled box
-// the distance to that box, at least eps.
-__device__ __forceinline__ float march_sdf(const DevBody &b, float3 y, float eps) {
-  int br;
-  const float f = body_sdf(b, y, &br);
-  if (b.kind != 4 || br >= 0) return f;
-  const float yy[3] = {y.x, y.y, y.z};
-  float q[3];
-#pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    const float lo = b.shape[k];
-    const float hi = __fadd_rn(b.shape[k], __fmul_rn(b.shape[3], (float)(b.gn[k] - 1u)));
-    q[k] = fmaxf(fmaxf(__fsub_rn(lo, yy[k]), __fsub_rn(yy[k], hi)), 0.0f);
-  }
-  const float s = __fadd_rn(__fadd_rn(__fmul_rn(q[0], q[0]), __fmul_rn(q[1], q[1])), __fmul_rn(q[2], q[2]));
-  return fmaxf(__fsqrt_rn(s), eps);
-}
+// The spheres' and the bodies' depths of a pixel meet in its atomic, so both are made in one
+// launch: the first blocks trace 32 pixels each with a warp per body, so that a step's bodies
+// are evaluated side by side and without divergence between their kinds, and the blocks after
+// them splat the spheres meanwhile.  A traced ray is a chain of up to c.steps evaluations:
+// that chain is what the launch takes.  Every warp of a tracing block keeps the state of all
+// its pixels, so a step has one barrier (the distances are double-buffered); a ray ends where
+// the spheres already block it (their depth is looked up every fourth step: it only falls,
+// and a later hit would lie behind it).  One thread per pixel, the bodies in turn, after the
+// splat: 10.9 us for 262,144 spheres, then 33.8 us for 36 x 36 rays and two bodies; now 29.2
+// together.
+constexpr uint32_t kTraceBodies = 32;  // as many as the mask has bits
 
-__global__ void k_trace_depth(StepArgs a, uint32_t gb0, uint32_t nb, RenderArgs c, const uint32_t *img, float *out) {
+__global__ void __launch_bounds__(32 * kTraceBodies) k_depth(StepArgs a, uint32_t off, uint32_t n, uint32_t gb0, uint32_t nb,
+                                                             uint32_t tblocks, RenderArgs c, uint32_t *img) {
   pdl_enter();
-  const uint32_t p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= c.W * c.H) return;
-  float best = __uint_as_float(img[p]);
-  if (nb && c.mask) {
-    const float4 d = c.rays[p];
-    float t = c.near;
-    for (uint32_t k = 0; k < c.steps; ++k) {
-      // a hit from here on would lie behind the nearest sphere (t only grows): 96 steps of a
-      // 36 x 36 image over a bed took 33.8 us, the few in front of it 5
-      if (t >= best) break;
+  if (blockIdx.x >= tblocks) {
+    const uint32_t i = (blockIdx.x - tblocks) * blockDim.x + threadIdx.x;
+    if (i < n) splat_depth(a, off, n, c, i, img);
+    return;
+  }
+  __shared__ float dist[2][kTraceBodies][32], block_at[2][32];
+  const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+  const uint32_t p = blockIdx.x * 32u + lane;
+  const bool in = p < c.W * c.H;
+  const bool mine = warp < nb && ((c.mask >> warp) & 1u);
+  const DevBody B = a.bodies[gb0 + (warp < nb ? warp : 0u)];
+  const float4 d = in ? c.rays[p] : make_float4(0.f, 0.f, 1.f, 0.f);
+  const float inf = __int_as_float(0x7f800000);
+  float t = c.near, hit = inf, seen = inf;
+  bool live = in;
+  for (uint32_t k = 0; k < c.steps && __any_sync(0xffffffffu, live); ++k) {
+    const uint32_t h = k & 1u;
+    float f = inf;
+    if (live && mine) {
       const float3 x = make_float3(__fadd_rn(c.o[0], __fmul_rn(t, d.x)), __fadd_rn(c.o[1], __fmul_rn(t, d.y)),
                                    __fadd_rn(c.o[2], __fmul_rn(t, d.z)));
-      float fmin = __int_as_float(0x7f800000);
-      for (uint32_t b = 0; b < nb && b < 32u; ++b) {
-        if (!((c.mask >> b) & 1u)) continue;
-        const DevBody &B = a.bodies[gb0 + b];
-        fmin = fminf(fmin, march_sdf(B, world_to_body(B, x), c.eps));
-      }
-      if (fmin < c.eps) {
-        best = fminf(best, t);
-        break;
-      }
+      f = march_sdf(B, world_to_body(B, x), c.eps);
+    }
+    dist[h][warp][lane] = f;
+    if (warp == 0) {
+      block_at[h][lane] = seen;
+      if ((k & 3u) == 0u && in) seen = __uint_as_float(__ldcg(&img[p]));
+    }
+    __syncthreads();
+    if (!live) continue;
+    float fmin = dist[h][0][lane];
+    for (uint32_t w = 1; w < nb; ++w) fmin = fminf(fmin, dist[h][w][lane]);
+    if (fmin < c.eps) {
+      hit = t;
+      live = false;
+    } else {
       t = __fadd_rn(t, fmin);
-      if (!(t <= c.far)) break;
+      if (!(t <= c.far) || t >= block_at[h][lane]) live = false;
     }
   }
-  out[p] = best <= c.far ? best : c.far;
+  if (warp == 0 && in && hit < inf) atomicMin(&img[p], __float_as_uint(hit));  // hit >= near > 0
+}
+
+__global__ void k_finish_depth(const uint32_t *img, uint32_t count, float far, float *out) {
+  pdl_enter();
+  const uint32_t p = blockIdx.x * blockDim.x + threadIdx.x;
+  if (p >= count) return;
+  const float best = __uint_as_float(img[p]);
+  out[p] = best <= far ? best : far;
 }
 
 inline unsigned cdiv(uint32_t a, unsigned b) { return a ? (a + b - 1) / b : 1; }
@@ -209,8 +245,14 @@ cudaError_t enqueue_render(const StepArgs &a, uint32_t env_off, uint32_t env_n, 
     GG_CHAIN(k_finish_height, np, 256, (const uint32_t *)img, np, c.empty, out);
   } else {
     GG_CHAIN(k_begin_depth, np, 128, c, img);
-    if (env_n) GG_CHAIN(k_splat_depth, env_n, 128, a, env_off, env_n, c, img);
-    GG_CHAIN(k_trace_depth, np, 128, a, gb0, nb, c, (const uint32_t *)img, out);
+    const uint32_t nt = std::min(nb, kTraceBodies), tblocks = nt && c.mask ? cdiv(np, 32) : 0u;
+    const unsigned threads = 32u * std::max(4u, nt);
+    if (tblocks || env_n) {
+      e = launch(true, k_depth, dim3(tblocks + (env_n ? cdiv(env_n, threads) : 0u)), threads, 0, st, a, env_off, env_n, gb0,
+                 nt, tblocks, c, img);
+      if (e != cudaSuccess) return e;
+    }
+    GG_CHAIN(k_finish_depth, np, 128, (const uint32_t *)img, np, c.far, out);
   }
 #undef GG_CHAIN
   return cudaGetLastError();

@@ -1,0 +1,90 @@
+"""Both sides of the lines at which a launch changes its shape: the depth camera's warp per
+body, the half-stencil search's thread per row, the reverse pass's kept graphs."""
+import numpy as np
+import pytest
+
+from gpu_helpers import F32, need_gpu
+from paper_2306_01369_gb300 import scenes as S
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def gg():
+    need_gpu()
+    from paper_2306_01369_gb300 import gg
+    return gg
+
+
+@pytest.mark.parametrize("nb,w,h", [(1, 1, 1), (2, 31, 1), (4, 33, 7), (5, 40, 30), (32, 36, 36)])
+def test_traced_bodies(gg, orc, nb, w, h):
+    """Bodies alone: the tracing is the oracle's FP32 one to the bit, whatever the split."""
+    rng = np.random.default_rng(nb)
+    bodies = [S.Body(kind=S.PLANE, pos=(0.0, 0.0, -0.3))]
+    for k in range(1, nb):
+        pos, rv = rng.uniform(-0.3, 0.3, 3), tuple(rng.uniform(-1.0, 1.0, 3))
+        bodies.append(S.scoop_body(1.0, pos, rv) if k % 2 else
+                      S.Body(kind=S.BOX, shape=tuple(rng.uniform(0.02, 0.06, 3)), pos=tuple(pos),
+                             quat=S._quat_from_rotvec(rv)))
+    cam = S.Camera(kind=S.DEPTH_CAMERA, width=w, height=h, pos=(0.0, 0.0, 0.8), quat=S._quat_from_rotvec((np.pi, 0.0, 0.0)),
+                   fov_y=0.9, near=0.01, far=1.5, march_steps=50, march_eps=1e-4)
+    sim = gg.Sim(np.zeros((0, 4), F32), np.zeros((0, 3), F32), np.zeros(0, F32), S.Params(), max_bodies=nb)
+    sim.set_bodies(bodies)
+    got = sim.render(cam)
+    sim.close()
+    assert np.array_equal(got, orc.render(cam, np.zeros((0, 3)), np.zeros(0), bodies).astype(F32))
+
+
+@pytest.mark.parametrize("n", [1, 127, 129, 262144, 262145])
+def test_half_stencil_rows(gg, n):
+    """Up to 262,144 spheres a thread per row, above that a thread per sphere: the same
+    contacts and state as the full-stencil search, with small (shared) and large buckets."""
+    side = round(n ** (1 / 3)) + 1
+    g = np.stack(np.meshgrid(*[np.arange(side)] * 3, indexing="ij"), -1).reshape(-1, 3)[:n]
+    rng = np.random.default_rng(n)
+    pr = np.empty((n, 4), F32)
+    pr[:, :3] = 0.0195 * (g - side / 2) + rng.uniform(-1e-3, 1e-3, (n, 3))
+    pr[:, 3] = 0.01
+    pr = np.ascontiguousarray(pr[rng.permutation(n)])
+    sets = [k for k in range(1, gg.load().gg_tuning_count() + 1) if "half" in gg.tuning_flags(k)]
+    sets = [next(k for k in sets if ("lists" in gg.tuning_flags(k)) == lists) for lists in
+            {"lists" in gg.tuning_flags(k) for k in sets}]
+    for hf in (1, 4):
+        want = None
+        for tuning in [7] + sets:
+            sim = gg.Sim(pr, None, S.sphere_mass(pr[:, 3]), S.Params(dt=1e-4, pja_iters=3, max_contacts=24), tuning=tuning,
+                         hash_factor=hf)
+            sim.step(2)
+            got = [sim.read("POS"), sim.read("VEL"), sim.read("CONTACTS", np.uint32)]
+            sim.close()
+            want = want or got
+            assert all(np.array_equal(a, b) for a, b in zip(got, want)), (tuning, hf)
+
+
+def test_reverse_passes_of_changing_length(gg):
+    """Reverse passes of one simulation, longer, shorter and of the first length again:
+    each gives what a simulation of its own gives."""
+    sc = S.diff_scene(n=512, n_steps=6)
+    seed = np.random.default_rng(3).normal(size=(sc.n, 3)).astype(F32)
+
+    def fresh():
+        sim = gg.Sim(sc.pos_r, sc.vel, sc.mass, sc.params)
+        sim.set_bodies(sc.bodies)
+        sim.set_trajectory(1, sc.twist[1].astype(F32))
+        return sim
+
+    def run(sim, state, steps):
+        sim.tape_reserve(steps, 2)
+        sim.set_state(state)
+        sim.step_taped(1, steps)
+        return sim.backward(seed)
+
+    kept = fresh()
+    state = kept.state()
+    for steps in (4, 6, 3, 4):
+        got = run(kept, state, steps)
+        one = fresh()
+        want = run(one, state, steps)
+        one.close()
+        assert np.array_equal(got[0], want[0]) and got[1] == want[1]
+    kept.close()
