@@ -648,7 +648,14 @@ __device__ __forceinline__ void mirror_pair(const StepArgs &a, uint32_t i, uint3
   if (aj < a.K) a.pscr[(size_t)(a.K + aj) * a.n + j] = i;
 }
 
+template <bool SPLIT>
 __device__ __forceinline__ void record_pair(const StepArgs &a, uint32_t i, uint32_t j, uint32_t &nf, uint32_t *jd) {
+  if (SPLIT) {
+    const uint32_t ai = atomicAdd(&a.pcnt[i], 0x10000u) >> 16;
+    mirror_pair(a, i, j);
+    if (ai < a.K) a.pscr[(size_t)ai * a.n + i] = j;
+    return;
+  }
   if (nf < a.K) a.pscr[(size_t)nf * a.n + i] = j;
   if (nf < kDeferPairs)
     jd[nf * kContactsBlock] = j;
@@ -669,7 +676,12 @@ __device__ __forceinline__ void mirror_deferred(const StepArgs &a, uint32_t i, u
     if (aj[q] < a.K) a.pscr[(size_t)(a.K + aj[q]) * a.n + j[q]] = i;
 }
 
-template <bool LISTS>
+// SPLIT: a thread per row of a particle (grid y), for particle counts that leave most of the
+// chip idle with a thread per particle: the five rows, each a chain of two or three
+// dependent loads, are then walked side by side, and the finder's slots come from the
+// counter too.
+constexpr int kRows = 5;
+template <bool LISTS, bool SPLIT>
 __global__ void __launch_bounds__(kContactsBlock, 9) k_pairs_half(StepArgs a) {
   pdl_enter();
   const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -718,7 +730,7 @@ __global__ void __launch_bounds__(kContactsBlock, 9) k_pairs_half(StepArgs a) {
   // rows (qy, qz) of the forward half, index 1 = offset 0: (0..2, 2) whole, (2, 1) whole,
   // (1, 1) with qx = 1 (the own cell) and 2
 #pragma unroll 1
-  for (int row = 0; row < 5; ++row) {
+  for (int row = SPLIT ? (int)blockIdx.y : 0; row < (SPLIT ? (int)blockIdx.y + 1 : kRows); ++row) {
     const int qz = row < 3 ? 2 : 1;
     const int qy = row < 3 ? row : (row == 3 ? 2 : 1);
     const uint32_t mask = row == 4 ? 6u : 7u;
@@ -761,7 +773,7 @@ __global__ void __launch_bounds__(kContactsBlock, 9) k_pairs_half(StepArgs a) {
           float d2;
           float3 d;
           const bool own = row == 4 && q == 1;
-          if ((own ? j > i : j != i) && sphere_hit(pi, pc[q], &d2, &d)) record_pair(a, i, j, nf, jd);
+          if ((own ? j > i : j != i) && sphere_hit(pi, pc[q], &d2, &d)) record_pair<SPLIT>(a, i, j, nf, jd);
           jn[q] = nx[q];
         }
       }
@@ -802,11 +814,12 @@ __global__ void __launch_bounds__(kContactsBlock, 9) k_pairs_half(StepArgs a) {
           r0[q] += (live >> q) & 1u;
           if (!((hit >> q) & 1u)) continue;
           const bool own = row == 4 && q == 1;
-          if (own ? jc[q] > i : jc[q] != i) record_pair(a, i, jc[q], nf, jd);
+          if (own ? jc[q] > i : jc[q] != i) record_pair<SPLIT>(a, i, jc[q], nf, jd);
         }
       }
     }
   }
+  if (SPLIT) return;
   mirror_deferred(a, i, nf, jd);
   if (nf) atomicAdd(&a.pcnt[i], min(nf, a.K + 1u) << 16);
 }
@@ -1440,6 +1453,14 @@ __global__ void k_body_state(const DevBody *bodies, uint32_t nbt, float *out) {
 // launchers
 // ---------------------------------------------------------------------------
 
+// Particle count up to which the half-stencil pass takes a thread per row.  Contact stage
+// (both passes) with a thread per particle and per row: 4,096 spheres 26.6 and 20.5 us,
+// 50,000 34.1 and 26.8, a pile of 262,144 68.9 and 64.1; 1,000,000 234 and 238, a batch of
+// 1.8 million 421 and 470 (the chip is full either way, and the extra atomics cost).  The
+// finder's share of pcnt cannot run over its 16 bits: 14 buckets of at most kMaxBucket.
+constexpr uint32_t kSplitRows = 262144;
+static_assert(14u * kMaxBucket < 65536u, "a row thread counts its hits in 16 bits");
+
 static inline unsigned grid_for(uint32_t n, int bs) { return (n + bs - 1) / bs > 0 ? (n + bs - 1) / bs : 1; }
 
 static inline cudaError_t mark(cudaEvent_t *ev, int k, cudaStream_t st) {
@@ -1521,10 +1542,18 @@ cudaError_t enqueue_step(const StepArgs &args, const LaunchShape &ls, cudaStream
     const size_t smem = (size_t)a.K * kContactsBlock * sizeof(uint32_t);
     const dim3 g(grid_for(a.n, kContactsBlock));
     if (ls.half) {
-      if (a.lists)
-        GG_LAUNCH(k_pairs_half<true>, g, kContactsBlock, 0, a);
-      else
-        GG_LAUNCH(k_pairs_half<false>, g, kContactsBlock, 0, a);
+      const dim3 gs(g.x, kRows);
+      if (a.n <= kSplitRows) {
+        if (a.lists)
+          GG_LAUNCH((k_pairs_half<true, true>), gs, kContactsBlock, 0, a);
+        else
+          GG_LAUNCH((k_pairs_half<false, true>), gs, kContactsBlock, 0, a);
+      } else {
+        if (a.lists)
+          GG_LAUNCH((k_pairs_half<true, false>), g, kContactsBlock, 0, a);
+        else
+          GG_LAUNCH((k_pairs_half<false, false>), g, kContactsBlock, 0, a);
+      }
       GG_LAUNCH(k_pairs_finish, g, kContactsBlock, smem, a);
     } else if (a.lists) {
       GG_LAUNCH(k_contacts<true>, g, kContactsBlock, smem, a);
