@@ -789,7 +789,7 @@ gg_status gg_create_batch(const gg_params *params, uint32_t n_envs, const uint32
       (rc = dalloc(s, &a.cn, nK)) || (rc = dalloc(s, &a.clam, 3 * nK)) || (rc = dalloc(s, &a.bj, nKb)) ||
       (rc = dalloc(s, &a.bn, nKb)) || (rc = dalloc(s, &a.bxc, nKb)) || (rc = dalloc(s, &a.blam, 3 * nKb)) ||
       (rc = dalloc(s, &a.envs, n_envs)) || (rc = dalloc(s, &a.bodies, nbt)) ||
-      (rc = dalloc(s, &a.chunk_env, chunks)) || (rc = dalloc(s, &a.wpart, (size_t)std::max(chunks, 1u) * s->maxb * 6)) ||
+      (rc = dalloc(s, &a.chunk, chunks)) || (rc = dalloc(s, &a.wpart, (size_t)std::max(chunks, 1u) * s->maxb * 6)) ||
       (rc = dalloc(s, &a.wrench, (size_t)s->H * nbt * 6)) || (rc = dalloc(s, &a.ctrl, 1)) ||
       (rc = dalloc(s, &s->vel3, (size_t)n * 3)) || (rc = dalloc(s, &a.ncb, nbt)) ||
       (rc = dalloc(s, &a.fcount, s->F)) || (rc = dalloc(s, &a.flist, (size_t)s->F * s->Lcap)) ||
@@ -824,9 +824,13 @@ gg_status gg_create_batch(const gg_params *params, uint32_t n_envs, const uint32
   a.F = s->F;
   a.Lcap = s->Lcap;
   s->fgb.assign(s->F, 0xffffffffu);
-  std::vector<uint32_t> h_chunk_env(std::max(chunks, 1u), 0);
+  std::vector<uint4> h_chunk(std::max(chunks, 1u));
   for (uint32_t e = 0; e < n_envs; ++e)
-    for (uint32_t c = 0; c < s->envs[e].nchunks; ++c) h_chunk_env[s->envs[e].chunk0 + c] = e;
+    for (uint32_t c = 0; c < s->envs[e].nchunks; ++c) {
+      const gg::DevEnv &E = s->envs[e];
+      const uint32_t first = E.off + c * gg::kWrenchChunk;
+      h_chunk[E.chunk0 + c] = make_uint4(e, first, std::min(first + gg::kWrenchChunk, E.off + E.n), 0);
+    }
   cudaError_t e;
 #define GG_UP(dst, src, bytes)                                                        \
   if ((e = cudaMemcpy((dst), (src), (bytes), cudaMemcpyHostToDevice)) != cudaSuccess) \
@@ -838,7 +842,7 @@ gg_status gg_create_batch(const gg_params *params, uint32_t n_envs, const uint32
   }
   GG_UP(wave_off, waves.data(), sizeof(uint32_t) * waves.size());
   GG_UP(a.envs, s->envs.data(), sizeof(DevEnv) * n_envs);
-  GG_UP(a.chunk_env, h_chunk_env.data(), sizeof(uint32_t) * h_chunk_env.size());
+  GG_UP(a.chunk, h_chunk.data(), sizeof(uint4) * h_chunk.size());
 #undef GG_UP
   if ((e = cudaMemset(a.cnt, 0, sizeof(uint32_t) * s->nh_cap)) != cudaSuccess ||
       (e = cudaMemset(a.start, 0, sizeof(uint32_t) * ((size_t)s->nh_cap + 4))) != cudaSuccess ||

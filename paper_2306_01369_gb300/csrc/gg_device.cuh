@@ -171,7 +171,7 @@ struct StepArgs {
   // environments and bodies
   DevEnv *envs;
   DevBody *bodies;
-  uint32_t *chunk_env;    // environment of each wrench chunk
+  uint4 *chunk;           // wrench chunks: environment, first particle, end
   float *wpart;           // [n_chunks][maxb][6]
   float *wrench;          // [wrench_hist][n_envs * maxb][6]
   DevCtrl *ctrl;

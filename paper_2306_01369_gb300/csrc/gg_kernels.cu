@@ -1164,23 +1164,25 @@ __device__ __forceinline__ void integrate_particle(const StepArgs &a, int s, uin
 //      each body's contact forces and torques over them in a fixed order
 // ---------------------------------------------------------------------------
 
-// One particle of the chunk per thread.  (Two per thread in 512-thread blocks, so that
-// a 262,144-sphere step's 256 chunks fit one wave of two blocks per SM, measured
-// slower: 16.0 against 14.3 us for the stage on the column.)
+// One particle of the chunk per thread.  The kernel waits for memory and for its barriers
+// (one block per SM), so it has one barrier for eight bodies: a warp without a contact with
+// a body adds nothing, and a thread per component adds the warps.  With two barriers and a
+// sum by one thread for every body the stage took 90 us for a batch of 1.8 million spheres,
+// 57 for 1 million, 11.9 for 4,096; now 52, 34 and 10.  (Chunks of 512 or 256: 49 and 49, 42
+// and 38, 9.8 and 9.8.)
 constexpr int kIntegrateThreads = kWrenchChunk;
+constexpr uint32_t kWrenchGroup = 8;  // bodies summed between two barriers
 
 __global__ void __launch_bounds__(kIntegrateThreads) k_integrate_wrench(StepArgs a, int s, int rev) {
   pdl_enter();
+  __shared__ float part[kWrenchGroup][kIntegrateThreads / 32][6];
   // rev: the last sweep ran forward in a serpentine launch shape, so start from the last
   // chunk, on the estimates still in L2 (the partials are per chunk: order changes nothing)
   const uint32_t c = rev ? gridDim.x - 1 - blockIdx.x : blockIdx.x;
-  const uint32_t e = a.chunk_env[c];
-  const DevEnv &E = a.envs[e];
-  const uint32_t s0 = E.off + (c - E.chunk0) * kWrenchChunk;
-  const uint32_t s1 = min(s0 + kWrenchChunk, E.off + E.n);
-  // one particle per thread (the chunk is the block)
-  const uint32_t i = s0 + threadIdx.x;
-  const bool own = i < s1;
+  const uint4 chunk = a.chunk[c];  // environment, particles [first, end)
+  const uint32_t i = chunk.y + threadIdx.x;
+  const bool own = i < chunk.z;
+  const uint32_t nbodies = a.envs[chunk.x].nbodies;
   const uint32_t nbc = own ? (a.ccount[i] >> 8) & 0xffu : 0u;
   if (own) integrate_particle(a, s, i);
   // linked-list binning: the step's lists have been walked, so empty every bucket for
@@ -1192,45 +1194,49 @@ __global__ void __launch_bounds__(kIntegrateThreads) k_integrate_wrench(StepArgs
     for (uint32_t b = blockIdx.x * kIntegrateThreads + threadIdx.x; b < a.nh_pad / 4u; b += gridDim.x * kIntegrateThreads)
       h4[b] = empty;
   }
-  // no body contact in the chunk (most chunks): every partial of the environment's
-  // bodies is zero, written at once (the partials of slot c are contiguous)
-  if (!__syncthreads_or(nbc != 0u)) {
-    for (uint32_t t = threadIdx.x; t < 6u * E.nbodies; t += kIntegrateThreads)
-      a.wpart[(size_t)c * a.maxb * 6 + t] = 0.f;
-    return;
-  }
   const size_t n = a.n, KbN = (size_t)a.Kb * n;
   const float inv_dt = 1.0f / a.dt;
-  for (uint32_t lb = 0; lb < E.nbodies; ++lb) {
-    const uint32_t gb = e * a.maxb + lb;
-    const DevBody &B = a.bodies[gb];
-    float v[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    int hit = 0;
-    for (uint32_t k = 0; k < nbc; ++k) {
-      const size_t o = (size_t)k * n + i;
-      if (a.bj[o] != gb) continue;
-      hit = 1;
-      const float fx = -a.blam[o] * inv_dt, fy = -a.blam[o + KbN] * inv_dt, fz = -a.blam[o + 2 * KbN] * inv_dt;
-      const float4 xc = a.bxc[o];
-      const float rx = xc.x - B.p[0], ry = xc.y - B.p[1], rz = xc.z - B.p[2];
-      v[0] += fx;
-      v[1] += fy;
-      v[2] += fz;
-      v[3] += ry * fz - rz * fy;
-      v[4] += rz * fx - rx * fz;
-      v[5] += rx * fy - ry * fx;
-    }
-    if (!__syncthreads_or(hit)) {  // no contact with this body in the chunk: zero partial
-      if (threadIdx.x < 6) a.wpart[((size_t)c * a.maxb + lb) * 6 + threadIdx.x] = 0.f;
-      continue;
-    }
-    block_sum6<kIntegrateThreads>(v);
-    if (threadIdx.x == 0) {
-      float *dst = a.wpart + ((size_t)c * a.maxb + lb) * 6;
+  const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, gb0 = chunk.x * a.maxb;
+  uint32_t k = 0, next = nbc ? a.bj[i] : 0xffffffffu;  // (a particle's bodies ascend)
+  for (uint32_t lb0 = 0; lb0 < nbodies; lb0 += kWrenchGroup) {
+    const uint32_t m = min(kWrenchGroup, nbodies - lb0);
+    if (lb0) __syncthreads();  // (the last group's sums are read)
+    for (uint32_t q = 0; q < m; ++q) {
+      const uint32_t gb = gb0 + lb0 + q;
+      float v[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+      const bool hit = next == gb;
+      if (hit) {
+        const size_t o = (size_t)k * n + i;
+        const float *p = a.bodies[gb].p;
+        const float fx = -a.blam[o] * inv_dt, fy = -a.blam[o + KbN] * inv_dt, fz = -a.blam[o + 2 * KbN] * inv_dt;
+        const float4 xc = a.bxc[o];
+        const float rx = xc.x - p[0], ry = xc.y - p[1], rz = xc.z - p[2];
+        v[0] += fx;
+        v[1] += fy;
+        v[2] += fz;
+        v[3] += ry * fz - rz * fy;
+        v[4] += rz * fx - rx * fz;
+        v[5] += rx * fy - ry * fx;
+        next = ++k < nbc ? a.bj[o + n] : 0xffffffffu;
+      }
+      if (__any_sync(0xffffffffu, hit)) {
 #pragma unroll
-      for (int k = 0; k < 6; ++k) dst[k] = v[k];
+        for (int d = 0; d < 6; ++d)
+#pragma unroll
+          for (int o = 16; o > 0; o >>= 1) v[d] += __shfl_xor_sync(0xffffffffu, v[d], o);
+      }
+      if (lane == 0)
+#pragma unroll
+        for (int d = 0; d < 6; ++d) part[q][warp][d] = v[d];
     }
-    __syncthreads();  // block_sum6's shared slots are reused by the next body
+    __syncthreads();
+    if (threadIdx.x < 6u * m) {  // the warps' sums in their order, a component a thread
+      const uint32_t q = threadIdx.x / 6u, d = threadIdx.x % 6u;
+      float t = part[q][0][d];
+#pragma unroll 8
+      for (int w = 1; w < kIntegrateThreads / 32; ++w) t += part[q][w][d];
+      a.wpart[((size_t)c * a.maxb + lb0) * 6 + threadIdx.x] = t;
+    }
   }
 }
 
@@ -1478,9 +1484,9 @@ __global__ void k_body_state(const DevBody *bodies, uint32_t nbt, float *out) {
 // ---------------------------------------------------------------------------
 
 // Particle count up to which the half-stencil pass takes a thread per row.  Contact stage
-// (both passes) with a thread per particle and per row: 4,096 spheres 26.6 and 20.5 us,
-// 50,000 34.1 and 26.8, a pile of 262,144 68.9 and 64.1; 1,000,000 234 and 238, a batch of
-// 1.8 million 421 and 470 (the chip is full either way, and the extra atomics cost).  The
+// (both passes) with a thread per particle and per row: 4,096 spheres 26.5 and 21.0 us,
+// 50,000 34.7 and 25.7, a pile of 262,144 60.4 and 55.3; 1,000,000 196 and 202, a batch of
+// 1.8 million 313 and 361 (the chip is full either way, and the extra atomics cost).  The
 // finder's share of pcnt cannot run over its 16 bits: 14 buckets of at most kMaxBucket.
 constexpr uint32_t kSplitRows = 262144;
 static_assert(14u * kMaxBucket < 65536u, "a row thread counts its hits in 16 bits");
