@@ -786,7 +786,7 @@ gg_status gg_create_batch(const gg_params *params, uint32_t n_envs, const uint32
       (rc = dalloc(s, &a.start, (size_t)s->nh_cap + 4)) || (rc = dalloc(s, &a.range, s->nh_cap)) || (rc = dalloc(s, &a.bsum, s->nh_cap / gg::kScanTile)) ||
       (rc = dalloc(s, &a.sid_tmp, n)) || (rc = dalloc(s, &a.sid, n)) || (rc = dalloc(s, &a.pos_s, n)) || (rc = dalloc(s, &a.U[0], n)) ||
       (rc = dalloc(s, &a.U[1], n)) || (rc = dalloc(s, &a.ccount, n)) || (rc = dalloc(s, &a.cj, nK)) ||
-      (rc = dalloc(s, &a.cn, nK)) || (rc = dalloc(s, &a.clam, 3 * nK)) || (rc = dalloc(s, &a.bj, nKb)) ||
+      (rc = dalloc(s, &a.cn, nK)) || (rc = dalloc(s, &a.clam, nK)) || (rc = dalloc(s, &a.bj, nKb)) ||
       (rc = dalloc(s, &a.bn, nKb)) || (rc = dalloc(s, &a.bxc, nKb)) || (rc = dalloc(s, &a.blam, 3 * nKb)) ||
       (rc = dalloc(s, &a.envs, n_envs)) || (rc = dalloc(s, &a.bodies, nbt)) ||
       (rc = dalloc(s, &a.chunk, chunks)) || (rc = dalloc(s, &a.wpart, (size_t)std::max(chunks, 1u) * s->maxb * 6)) ||

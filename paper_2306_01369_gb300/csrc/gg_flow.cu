@@ -161,7 +161,7 @@ __device__ __forceinline__ void hand_over(const StepArgs &a, uint32_t fid, size_
 __device__ __forceinline__ void barrier_sweeps(const StepArgs &a, uint32_t iters, uint32_t G, uint32_t p0, uint32_t p1) {
   const Tape none{};
   const uint32_t stride = G * kFlowThreads;
-  const size_t n = a.n, KN = (size_t)a.K * n, KbN = (size_t)a.Kb * n;
+  const size_t n = a.n, KbN = (size_t)a.Kb * n;
   if (blockIdx.x < G)
     for (uint32_t i = p0 + blockIdx.x * kFlowThreads + threadIdx.x; i < p1; i += stride) {
       const uint32_t cc = a.ccount[i];
@@ -169,7 +169,7 @@ __device__ __forceinline__ void barrier_sweeps(const StepArgs &a, uint32_t iters
         const float4 b = base_velocity(a, a.vel_id[i]);
         a.U[0][i] = make_float4(b.x, b.y, b.z, a.lit ? b.w : 0.f);
       }
-      for (uint32_t c = 0; c < 3 * (cc & 0xffu); ++c) a.clam[(size_t)(c % 3) * KN + (size_t)(c / 3) * n + i] = 0.f;
+      for (uint32_t c = 0; c < (cc & 0xffu); ++c) a.clam[(size_t)c * n + i] = no_impulse(a.cj[(size_t)c * n + i]);
       for (uint32_t c = 0; c < 3 * ((cc >> 8) & 0xffu); ++c) a.blam[(size_t)(c % 3) * KbN + (size_t)(c / 3) * n + i] = 0.f;
     }
   grid_barrier(a.ctrl, a.wait_cycles);
@@ -416,11 +416,15 @@ __device__ __forceinline__ void sweeps(const StepArgs &a, const Block &k, uint32
       const uint32_t r = at<uint32_t>(ref, 32u * c);
       const float sg = (r & kSign) ? -1.f : 1.f;
       const float4 l = referred(a, r);
-      float *d = c < npp ? a.clam + (size_t)c * n + i : a.blam + (size_t)(c - npp) * n + i;
-      const size_t plane = (size_t)(c < npp ? a.K : a.Kb) * n;
-      d[0] = sg * l.x;
-      d[plane] = sg * l.y;
-      d[2 * plane] = sg * l.z;
+      if (c < npp) {
+        a.clam[(size_t)c * n + i] = make_float4(sg * l.x, sg * l.y, sg * l.z, 0.f);
+      } else {
+        float *d = a.blam + (size_t)(c - npp) * n + i;
+        const size_t plane = (size_t)a.Kb * n;
+        d[0] = sg * l.x;
+        d[plane] = sg * l.y;
+        d[2 * plane] = sg * l.z;
+      }
     }
   }
 }

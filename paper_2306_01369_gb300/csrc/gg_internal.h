@@ -33,7 +33,7 @@ struct LaunchShape {
   int fused_block;      // > 0: all sweeps in one cooperative launch of this block size ...
   uint32_t fused_grid;  // ... and this many blocks (all resident); 0: one launch per sweep
   uint32_t lists;       // binning: 0 counting sort, 1 linked list per bucket (Alg. 2)
-  uint32_t lean;        // per-launch sweeps capped at 40 registers (more resident warps: pays
+  uint32_t lean;        // per-launch sweeps capped at 56 registers (more resident warps: pays
                         // when the working set spills out of L2, costs when it fits)
   uint32_t half;        // pair search over half the stencil in two passes instead of k_contacts
   uint32_t detect;      // detection and all sweeps in one cooperative launch (fused_grid blocks)

@@ -365,9 +365,7 @@ __device__ __forceinline__ void contact_records(const StepArgs &a, uint32_t i, f
         a.cj[o] = j;
         a.cn[o] = g;
         if (a.flow) continue;  // (the dataflow sweeps start their impulses at zero themselves)
-        a.clam[o] = 0.f;
-        a.clam[o + (size_t)K * n] = 0.f;
-        a.clam[o + 2 * (size_t)K * n] = 0.f;
+        a.clam[o] = no_impulse(j);
       }
     }
     // particle-body contacts, bodies in ascending index
@@ -928,16 +926,18 @@ __global__ void __launch_bounds__(512) k_pja(StepArgs a, int s, Tape tp, int it,
   if (i < a.n) pja_particle<TAPE, false, PRE>(a, i, s, tp, it);
 }
 
-// One sweep per launch with at most 40 registers per thread (62.5 % -> 75 % occupancy
-// at 256-thread blocks, at the price of a few spilled values): the autotuner's choice
-// when the sweep's working set streams from DRAM.
-__global__ void __maxnreg__(40) k_pja_lean(StepArgs a, int s, int it, int rev) {
+// One sweep per launch with at most 56 registers per thread (nine blocks of 128 an SM
+// instead of eight, and nothing spilled): the autotuner's choice when the sweep's working
+// set streams from DRAM.  1M spheres, with the free bodies' update after each sweep: 48.2 us
+// a sweep at 40 registers and planar impulses, 44.1 at 56 and one 16-byte record of impulse
+// and partner (64: 45.7, 48: 45.3, 40: 48.8; computing the normal again from the positions
+// instead of reading it: 43.7 at 48 registers, 44.8 at 56, slower over the whole step).
+__global__ void __maxnreg__(56) k_pja_lean(StepArgs a, int s, int it, int rev) {
   pdl_enter();
   const uint32_t i = sweep_particle(rev);
   const Tape none{};
   if (i < a.n) pja_particle<false, false>(a, i, s, none, it);
 }
-
 
 // OneLoop, the third form of the paper's loop-structure ablation (Sec. II-D, Fig.
 // warp-divergence-performance): every impulse iteration walks the neighbour cells
@@ -963,8 +963,8 @@ __global__ void __launch_bounds__(kContactsBlock) k_oneloop(StepArgs a, int s) {
   bool ovf = false;
   walk_partners<LISTS>(a, i, pi, E, fid, S, npp, ovf);
   const float4 *__restrict__ Uin = a.U[s];
-  float *__restrict__ clam = a.clam;
-  const size_t n = a.n, KN = (size_t)a.K * n, KbN = (size_t)a.Kb * n;
+  float4 *__restrict__ clam = a.clam;
+  const size_t n = a.n, KbN = (size_t)a.Kb * n;
   const float4 ui = Uin[i];
   const float4 base = base_velocity(a, a.vel_id[i]);
   const float pw = a.lit ? 0.f : 1.f;
@@ -974,12 +974,11 @@ __global__ void __launch_bounds__(kContactsBlock) k_oneloop(StepArgs a, int s) {
     const float4 g = pair_geometry(pi, a.pos_id[j], i, j);
     const float4 uj = Uin[j];
     const size_t o = (size_t)c * n + i;
-    const float3 l = pja_project(make_float3(clam[o], clam[o + KN], clam[o + 2 * KN]),
+    const float4 la = clam[o];
+    const float3 l = pja_project(make_float3(la.x, la.y, la.z),
                                  make_float3(ui.x - uj.x, ui.y - uj.y, ui.z - uj.z), make_float3(g.x, g.y, g.z),
                                  a.ab * g.w, 1.0f / (ui.w + pw * uj.w), a.mu);
-    clam[o] = l.x;
-    clam[o + KN] = l.y;
-    clam[o + 2 * KN] = l.z;
+    clam[o] = make_float4(l.x, l.y, l.z, la.w);
     sx += l.x;
     sy += l.y;
     sz += l.z;
@@ -1414,9 +1413,10 @@ __global__ void k_export_contacts(StepArgs a, uint32_t *rows, float *geom, float
     }
     if (lam) {
       float *d = lam + ((size_t)id * K + c) * 3;
-      d[0] = on ? a.clam[o] : 0.f;
-      d[1] = on ? a.clam[o + (size_t)K * n] : 0.f;
-      d[2] = on ? a.clam[o + 2 * (size_t)K * n] : 0.f;
+      const float4 l = on ? a.clam[o] : make_float4(0.f, 0.f, 0.f, 0.f);
+      d[0] = l.x;
+      d[1] = l.y;
+      d[2] = l.z;
     }
   }
   for (uint32_t c = 0; c < Kb; ++c) {

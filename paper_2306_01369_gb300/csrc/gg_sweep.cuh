@@ -41,6 +41,9 @@ __device__ __forceinline__ void block_sum6(float v[6]) {
 
 __device__ __forceinline__ void flag(DevCtrl *c, uint32_t f) { atomicOr(&c->status, f); }
 
+// a contact's record before its first update: no impulse, the partner's id
+__device__ __forceinline__ float4 no_impulse(uint32_t j) { return make_float4(0.f, 0.f, 0.f, __uint_as_float(j)); }
+
 // v + dt g (the velocity before contact impulses), with 1/m in w; the fused multiply-add is
 // spelled out, so that a hoisted product cannot round differently in one of the callers
 __device__ __forceinline__ float4 base_velocity(const StepArgs &a, float4 v) {
@@ -55,9 +58,8 @@ __device__ __forceinline__ float4 base_velocity(const StepArgs &a, float4 v) {
 template <bool TAPE, bool LDCG, bool PRE = false>
 __device__ __forceinline__ void pja_particle(const StepArgs &a, uint32_t i, int s, const Tape &tp, int it) {
   const float4 *__restrict__ Uin = a.U[s];
-  const uint32_t *__restrict__ cj = a.cj;
   const float4 *__restrict__ cn = a.cn;
-  float *__restrict__ clam = a.clam;
+  float4 *__restrict__ clam = a.clam;
   const size_t n = a.n;
   const uint32_t cc = a.ccount[i];
   const uint32_t npp = cc & 0xffu, nbc = (cc >> 8) & 0xffu;
@@ -68,12 +70,10 @@ __device__ __forceinline__ void pja_particle(const StepArgs &a, uint32_t i, int 
   const float mu = a.mu, ab = a.ab;
   const float pw = a.lit ? 0.f : 1.f;  // partner's share of the effective mass (exact 0 or 1)
   // one contact update (Alg. 1 with the accumulated clamp): new impulse stored (and taped)
-  auto update = [&](size_t o, const float4 &nn, const float3 &la, const float4 &uj) {
-    const float3 l = pja_project(la, make_float3(ui.x - uj.x, ui.y - uj.y, ui.z - uj.z), make_float3(nn.x, nn.y, nn.z),
+  auto update = [&](size_t o, const float4 &nn, const float4 &la, const float4 &uj) {
+    const float3 l = pja_project(make_float3(la.x, la.y, la.z), make_float3(ui.x - uj.x, ui.y - uj.y, ui.z - uj.z), make_float3(nn.x, nn.y, nn.z),
                                  ab * nn.w, 1.0f / (ui.w + pw * uj.w), mu);
-    clam[o] = l.x;
-    clam[o + KN] = l.y;
-    clam[o + 2 * KN] = l.z;
+    clam[o] = make_float4(l.x, l.y, l.z, la.w);
     if (TAPE) {
       float *h = tp.lamh + (size_t)(it + 1) * 3 * KN;
       h[o] = l.x;
@@ -93,24 +93,20 @@ __device__ __forceinline__ void pja_particle(const StepArgs &a, uint32_t i, int 
   // (Loading only the partner ids of slots 0 and 1 early was measured too: slower on
   // every workload, 64 registers with spills.)
   const bool two = PRE && a.K > 1;
-  uint32_t pj0 = 0u, pj1 = 0u;
-  float4 pn0 = make_float4(0.f, 0.f, 0.f, 0.f), pn1 = pn0;
-  float3 pl0 = make_float3(0.f, 0.f, 0.f), pl1 = pl0;
+  float4 pn0 = make_float4(0.f, 0.f, 0.f, 0.f), pn1 = pn0, pl0 = pn0, pl1 = pn0;
   if (PRE) {
-    pj0 = cj[i];
     pn0 = cn[i];
-    pl0 = make_float3(clam[i], clam[i + KN], clam[i + 2 * KN]);
+    pl0 = clam[i];
     if (two) {
-      pj1 = cj[n + i];
       pn1 = cn[n + i];
-      pl1 = make_float3(clam[n + i], clam[n + i + KN], clam[n + i + 2 * KN]);
+      pl1 = clam[n + i];
     }
   }
   // two contacts per round: both rounds' loads issue before either update is stored;
   // the impulses are still added in contact order
   uint32_t c = 0;
   if (two && npp >= 2) {
-    uint32_t j0 = pj0, j1 = pj1;
+    uint32_t j0 = __float_as_uint(pl0.w), j1 = __float_as_uint(pl1.w);
     if (!GG_GUARD(a.ctrl, j0 < a.n && j1 < a.n)) j0 = j1 = i;  // debug build: never gather out of range
     const float4 u0 = gather(j0), u1 = gather(j1);
     const float3 l0 = update(i, pn0, pl0, u0);
@@ -125,11 +121,10 @@ __device__ __forceinline__ void pja_particle(const StepArgs &a, uint32_t i, int 
   }
   for (; c + 1 < npp; c += 2) {
     const size_t o0 = (size_t)c * n + i, o1 = o0 + n;
-    uint32_t j0 = cj[o0], j1 = cj[o1];
-    if (!GG_GUARD(a.ctrl, j0 < a.n && j1 < a.n)) j0 = j1 = i;  // debug build: never gather out of range
     const float4 n0 = cn[o0], n1 = cn[o1];
-    const float3 la0 = make_float3(clam[o0], clam[o0 + KN], clam[o0 + 2 * KN]);
-    const float3 la1 = make_float3(clam[o1], clam[o1 + KN], clam[o1 + 2 * KN]);
+    const float4 la0 = clam[o0], la1 = clam[o1];
+    uint32_t j0 = __float_as_uint(la0.w), j1 = __float_as_uint(la1.w);
+    if (!GG_GUARD(a.ctrl, j0 < a.n && j1 < a.n)) j0 = j1 = i;  // debug build: never gather out of range
     const float4 u0 = gather(j0), u1 = gather(j1);
     const float3 l0 = update(o0, n0, la0, u0);
     const float3 l1 = update(o1, n1, la1, u1);
@@ -143,10 +138,10 @@ __device__ __forceinline__ void pja_particle(const StepArgs &a, uint32_t i, int 
   if (c < npp) {
     const size_t o = (size_t)c * n + i;
     const bool pre = PRE && c == 0;
-    uint32_t j = pre ? pj0 : cj[o];
+    const float4 lam = pre ? pl0 : clam[o];
+    uint32_t j = __float_as_uint(lam.w);
     if (!GG_GUARD(a.ctrl, j < a.n)) j = i;
     const float4 nn = pre ? pn0 : cn[o];
-    const float3 lam = pre ? pl0 : make_float3(clam[o], clam[o + KN], clam[o + 2 * KN]);
     const float3 l = update(o, nn, lam, gather(j));
     sx += l.x;
     sy += l.y;
