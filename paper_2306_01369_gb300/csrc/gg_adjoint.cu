@@ -135,14 +135,17 @@ __device__ __forceinline__ float3 rotT(const float *R, float3 v) {
                      R[2] * v.x + R[5] * v.y + R[8] * v.z);
 }
 
-// fixed-order block sum of kPart floats into part[blk][*]
-__device__ __forceinline__ void block_partials(float v[kPart], float *dst) {
+// fixed-order block sum of kPart floats into dst[*], or (ADD) added to what is there, with
+// the rounding error of the running sum carried along in dst[kPart + *]
+template <bool ADD>
+__device__ __forceinline__ void block_partials(float v[kPart], float *dst, bool first = true) {
   __shared__ float sm[kAdjThreads / 32][kPart];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
 #pragma unroll
   for (int k = 0; k < kPart; ++k)
+    if (__any_sync(0xffffffffu, v[k] != 0.f))  // (few warps touch the tool)
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
+      for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
   if (lane == 0)
 #pragma unroll
     for (int k = 0; k < kPart; ++k) sm[wid][k] = v[k];
@@ -150,7 +153,14 @@ __device__ __forceinline__ void block_partials(float v[kPart], float *dst) {
   if (threadIdx.x < kPart) {
     float s = sm[0][threadIdx.x];
     for (int w = 1; w < kAdjThreads / 32; ++w) s += sm[w][threadIdx.x];
+    float err = 0.f;
+    if (ADD && !first) {
+      const float x = dst[threadIdx.x], y = __fadd_rn(s, dst[kPart + threadIdx.x]);
+      s = __fadd_rn(x, y);
+      err = __fsub_rn(y, __fsub_rn(s, x));
+    }
     dst[threadIdx.x] = s;
+    if (ADD) dst[kPart + threadIdx.x] = err;
   }
 }
 
@@ -178,7 +188,7 @@ __global__ void __launch_bounds__(kAdjThreads) k_adj_begin(StepArgs a, AdjArgs d
   pdl_enter();
   const uint32_t s = blockIdx.x * blockDim.x + threadIdx.x;
   if (s >= a.n) return;
-  const size_t n = a.n, KN = (size_t)a.K * n, KbN = (size_t)a.Kb * n;
+  const size_t n = a.n, KbN = (size_t)a.Kb * n;
   const uint32_t id = s;
   const float4 xb = d.xbar[id], vb = d.vbar[id];
   d.xbar_s[s] = xb;
@@ -190,9 +200,8 @@ __global__ void __launch_bounds__(kAdjThreads) k_adj_begin(StepArgs a, AdjArgs d
   const float3 zero = make_float3(0.f, 0.f, 0.f);
   for (uint32_t c = 0; c < npp; ++c) {
     const size_t o = (size_t)c * n + s;
-    st3(d.Lbar, o, KN, zero);
-    st3(d.nbar, o, KN, zero);
-    d.psibar[o] = 0.f;
+    d.Lbar[o] = make_float4(0.f, 0.f, 0.f, 0.f);
+    d.nbar[o] = make_float4(0.f, 0.f, 0.f, 0.f);
   }
   for (uint32_t c = 0; c < nbc; ++c) {
     const size_t o = (size_t)c * n + s;
@@ -206,18 +215,18 @@ __global__ void __launch_bounds__(kAdjThreads) k_adj_begin(StepArgs a, AdjArgs d
 // Subtracts the twin contacts' u-bar (of the sweep whose u-bar is in `ub`) from U, the
 // own-contact part of a U-bar, and adds the completed U-bar to the base velocity's.
 __device__ __forceinline__ float4 complete_ubar(const StepArgs &a, const AdjArgs &d, uint32_t i, float4 U,
-                                                const float *ub) {
-  const size_t n = a.n, KN = (size_t)a.K * n;
+                                                const float4 *ub) {
+  const size_t n = a.n;
   const uint32_t npp = a.ccount[i] & 0xffu;
 #pragma unroll 4
   for (uint32_t c = 0; c < npp; ++c) {  // loads only: four contacts' gathers in flight
     const size_t o = (size_t)c * n + i;
     const uint32_t tw = d.twin[o], jt = a.cj[o];
     if (!GG_GUARD(a.ctrl, tw < a.K && jt < a.n)) continue;
-    const size_t ot = (size_t)tw * n + jt;
-    U.x -= ub[ot];
-    U.y -= ub[ot + KN];
-    U.z -= ub[ot + 2 * KN];
+    const float4 u = ub[(size_t)tw * n + jt];
+    U.x -= u.x;
+    U.y -= u.y;
+    U.z -= u.z;
   }
   const float4 b = d.basebar[i];
   d.basebar[i] = make_float4(b.x + U.x, b.y + U.y, b.z + U.z, 0.f);
@@ -227,63 +236,77 @@ __device__ __forceinline__ float4 complete_ubar(const StepArgs &a, const AdjArgs
 // Reverse of sweep s (U^s, lambda^s -> lambda^{s+1}, U^{s+1}).  Ubar[cur] holds the
 // own-contact part of the adjoint of U^{s+1} (complete for s + 1 = I); the own-contact
 // part of the adjoint of U^s goes to Ubar[cur ^ 1], this sweep's u-bar to ubar[s & 1].
-__global__ void __launch_bounds__(kAdjThreads) k_adj_iter(StepArgs a, AdjArgs d, uint32_t s, int cur) {
+// G lanes a particle, a contact each: a contact's reverse is a long chain of dependent
+// instructions, and a thread that took its particle's contacts in turn left a bed of 32,768
+// spheres with two warps a scheduler to hide them.  The sums over a particle's contacts are
+// still added in contact order.
+constexpr uint32_t kFull = 0xffffffffu;
+
+template <int G>
+__global__ void __launch_bounds__(kAdjThreads, 4) k_adj_iter(StepArgs a, AdjArgs d, uint32_t s, int cur) {
   pdl_enter();
-  const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+  const uint32_t i = (blockIdx.x * kAdjThreads + threadIdx.x) / G, l = threadIdx.x % G;
+  const bool in = i < a.n;
   float part[kPart] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-  if (i < a.n) {
-    const size_t n = a.n, KN = (size_t)a.K * n, KbN = (size_t)a.Kb * n;
-    float4 Un = d.Ubar[cur][i];
-    if (s + 1 < d.I) Un = complete_ubar(a, d, i, Un, d.ubar[(s + 1) & 1u]);
-    float *ubar = d.ubar[s & 1u];
-    const float invm = a.vel_id[i].w;
-    const float4 Ui = d.tp.Uh[(size_t)s * n + i];
-    const float *lh = d.tp.lamh + (size_t)s * 3 * KN;
-    const float *blh = d.tp.blamh + (size_t)s * 3 * KbN;
-    const uint32_t cc = a.ccount[i];
-    const uint32_t npp = cc & 0xffu, nbc = (cc >> 8) & 0xffu;
-    float3 S = make_float3(0.f, 0.f, 0.f);
-    float mub = 0.f;
-    // Reverse of one contact update, from its loaded inputs; stores its adjoints.
-    const float4 *Uh = d.tp.Uh + (size_t)s * n;
-    auto contact = [&](size_t o, float4 nn, float3 lam, float3 Lb, float psb, float3 nbo, float4 Uj) {
-      const float3 nv = f3(nn);
-      const float w = 1.0f / (Ui.w + Uj.w);
-      const float bias = a.ab * nn.w;
-      const float3 z = pja_pre(lam, make_float3(Ui.x - Uj.x, Ui.y - Uj.y, Ui.z - Uj.z), nv, bias, w);
-      const float3 abar = add(mul(invm, f3(Un)), Lb);
-      float3 nb = make_float3(0.f, 0.f, 0.f);
-      const float3 zb = cone_adjoint(z, nv, a.mu, abar, &nb, &mub);
-      st3(d.Lbar, o, KN, zb);
-      const float3 ub = mul(-w, zb);
-      st3(ubar, o, KN, ub);
-      S = add(S, ub);
-      d.psibar[o] = psb + w * a.ab * dot(nv, zb);
-      st3(d.nbar, o, KN, add(nbo, add(mul(w * bias, zb), nb)));
-    };
-    // two contacts per round: both contacts' loads are issued before either's stores
-    uint32_t c = 0;
-    for (; c + 1 < npp; c += 2) {
-      const size_t o0 = (size_t)c * n + i, o1 = o0 + n;
-      uint32_t j0 = a.cj[o0], j1 = a.cj[o1];
-      if (!GG_GUARD(a.ctrl, j0 < a.n && j1 < a.n)) j0 = j1 = i;
-      const float4 nn0 = a.cn[o0], nn1 = a.cn[o1];
-      const float3 lm0 = ld3(lh, o0, KN), lm1 = ld3(lh, o1, KN);
-      const float3 Lb0 = ld3(d.Lbar, o0, KN), Lb1 = ld3(d.Lbar, o1, KN);
-      const float ps0 = d.psibar[o0], ps1 = d.psibar[o1];
-      const float3 nb0 = ld3(d.nbar, o0, KN), nb1 = ld3(d.nbar, o1, KN);
-      const float4 Uj0 = Uh[j0], Uj1 = Uh[j1];
-      contact(o0, nn0, lm0, Lb0, ps0, nb0, Uj0);
-      contact(o1, nn1, lm1, Lb1, ps1, nb1, Uj1);
+  const size_t n = a.n, KN = (size_t)a.K * n, KbN = (size_t)a.Kb * n;
+  const uint32_t cc = in ? a.ccount[i] : 0u;
+  const uint32_t npp = cc & 0xffu, tot = npp + ((cc >> 8) & 0xffu);
+  float4 Un = make_float4(0.f, 0.f, 0.f, 0.f), Ui = Un;
+  float invm = 0.f;
+  if (in) {
+    Un = d.Ubar[cur][i];
+    Ui = d.tp.Uh[(size_t)s * n + i];
+    invm = a.vel_id[i].w;
+  }
+  const uint32_t most = __reduce_max_sync(kFull, tot);  // rounds are the warp's
+  if (s + 1 < d.I) {  // the twins' u-bar of the sweep after completes U-bar^{s+1}
+    const float4 *ub = d.ubar[(s + 1) & 1u];
+    for (uint32_t c0 = 0; c0 < most; c0 += G) {
+      float4 u = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (c0 + l < npp) {
+        const size_t o = (size_t)(c0 + l) * n + i;
+        const uint32_t tw = d.twin[o], jt = a.cj[o];
+        if (GG_GUARD(a.ctrl, tw < a.K && jt < a.n)) u = ub[(size_t)tw * n + jt];
+      }
+#pragma unroll
+      for (int q = 0; q < G; ++q) {
+        Un.x -= __shfl_sync(kFull, u.x, q, G);
+        Un.y -= __shfl_sync(kFull, u.y, q, G);
+        Un.z -= __shfl_sync(kFull, u.z, q, G);
+      }
     }
+    if (in && l == 0) {
+      const float4 b = d.basebar[i];
+      d.basebar[i] = make_float4(b.x + Un.x, b.y + Un.y, b.z + Un.z, 0.f);
+    }
+  }
+  const float4 *Uh = d.tp.Uh + (size_t)s * n;
+  float3 S = make_float3(0.f, 0.f, 0.f);
+  float mub = 0.f;
+  for (uint32_t c0 = 0; c0 < most; c0 += G) {
+    const uint32_t c = c0 + l;
+    float3 ub = make_float3(0.f, 0.f, 0.f);  // the contact's share of S ...
+    float mu = 0.f;                          // ... and of mu's adjoint
     if (c < npp) {
       const size_t o = (size_t)c * n + i;
       uint32_t j = a.cj[o];
       if (!GG_GUARD(a.ctrl, j < a.n)) j = i;
-      contact(o, a.cn[o], ld3(lh, o, KN), ld3(d.Lbar, o, KN), d.psibar[o], ld3(d.nbar, o, KN), Uh[j]);
-    }
-    for (uint32_t c = 0; c < nbc; ++c) {
-      const size_t o = (size_t)c * n + i;
+      const float4 nn = a.cn[o], Lb = d.Lbar[o], nbo = d.nbar[o], Uj = Uh[j];
+      const float3 lam = ld3(d.tp.lamh + (size_t)s * 3 * KN, o, KN);
+      const float3 nv = f3(nn);
+      const float w = 1.0f / (Ui.w + Uj.w);
+      const float bias = a.ab * nn.w;
+      const float3 z = pja_pre(lam, make_float3(Ui.x - Uj.x, Ui.y - Uj.y, Ui.z - Uj.z), nv, bias, w);
+      const float3 abar = add(mul(invm, f3(Un)), f3(Lb));
+      float3 nb = make_float3(0.f, 0.f, 0.f);
+      const float3 zb = cone_adjoint(z, nv, a.mu, abar, &nb, &mu);
+      d.Lbar[o] = make_float4(zb.x, zb.y, zb.z, Lb.w + w * a.ab * dot(nv, zb));  // (w: psi-bar)
+      ub = mul(-w, zb);
+      d.ubar[s & 1u][o] = make_float4(ub.x, ub.y, ub.z, 0.f);
+      const float3 no = add(f3(nbo), add(mul(w * bias, zb), nb));
+      d.nbar[o] = make_float4(no.x, no.y, no.z, 0.f);
+    } else if (c < tot) {
+      const size_t o = (size_t)(c - npp) * n + i;
       const uint32_t gb = a.bj[o];
       const DevBody &B = a.bodies[gb];
       const float4 nn = a.bn[o];
@@ -294,16 +317,15 @@ __global__ void __launch_bounds__(kAdjThreads) k_adj_iter(StepArgs a, AdjArgs d,
       const float3 ubody = add(make_float3(B.v[0], B.v[1], B.v[2]), cross(W, r));
       const float w = 1.0f / Ui.w;
       const float bias = a.ab * nn.w;
-      const float3 z = pja_pre(ld3(blh, o, KbN), sub(f3(Ui), ubody), nv, bias, w);
+      const float3 z = pja_pre(ld3(d.tp.blamh + (size_t)s * 3 * KbN, o, KbN), sub(f3(Ui), ubody), nv, bias, w);
       const float3 abar = add(mul(invm, f3(Un)), ld3(d.bLbar, o, KbN));
       float3 nb = make_float3(0.f, 0.f, 0.f);
-      const float3 zb = cone_adjoint(z, nv, a.mu, abar, &nb, &mub);
+      const float3 zb = cone_adjoint(z, nv, a.mu, abar, &nb, &mu);
       st3(d.bLbar, o, KbN, zb);
-      const float3 uu = mul(-w, zb);  // adjoint of u = U_i - u_body
-      S = add(S, uu);
+      ub = mul(-w, zb);  // adjoint of u = U_i - u_body
       d.bpsibar[o] += w * a.ab * dot(nv, zb);
       acc3(d.bnbar, o, KbN, add(mul(w * bias, zb), nb));
-      const float3 ubb = mul(-1.f, uu);  // adjoint of the body point velocity
+      const float3 ubb = mul(-1.f, ub);  // adjoint of the body point velocity
       acc3(d.bxcbar, o, KbN, mul(-1.f, cross(W, ubb)));  // u_body = V + W x (x_c - p)
       if (gb == d.tool) {
         const float3 wr = cross(r, ubb), pw = cross(W, ubb);
@@ -318,20 +340,30 @@ __global__ void __launch_bounds__(kAdjThreads) k_adj_iter(StepArgs a, AdjArgs d,
         part[8] += pw.z;
       }
     }
-    part[9] = mub;
-    d.Ubar[cur ^ 1][i] = make_float4(S.x, S.y, S.z, 0.f);
+#pragma unroll
+    for (int q = 0; q < G; ++q) {
+      S.x += __shfl_sync(kFull, ub.x, q, G);
+      S.y += __shfl_sync(kFull, ub.y, q, G);
+      S.z += __shfl_sync(kFull, ub.z, q, G);
+      mub += __shfl_sync(kFull, mu, q, G);
+    }
   }
-  block_partials(part, d.part + ((size_t)s * d.nblk + blockIdx.x) * kPart);
+  if (l == 0) {
+    part[9] = mub;
+    if (in) d.Ubar[cur ^ 1][i] = make_float4(S.x, S.y, S.z, 0.f);
+  }
+  // (a block's sweeps follow one another, so its sum over them is kept, not one a sweep)
+  block_partials<true>(part, d.part + (size_t)blockIdx.x * 2 * kPart, s + 1 == d.I);
 }
 
 // gradient of a pair contact's psi and normal w.r.t. the particle's own position
-__device__ __forceinline__ float3 pair_geom_grad(const AdjArgs &d, const StepArgs &a, size_t o, size_t KN, float dist) {
+__device__ __forceinline__ float3 pair_geom_grad(const AdjArgs &d, const StepArgs &a, size_t o, float dist) {
   const float4 nn = a.cn[o];
   const float3 nv = f3(nn);
-  const float3 nb = ld3(d.nbar, o, KN);
+  const float3 nb = f3(d.nbar[o]);
   const float nbn = dot(nb, nv);
   const float id = dist > 0.f ? 1.0f / dist : 0.f;
-  return add(mul(-d.psibar[o], nv), mul(id, sub(nb, mul(nbn, nv))));
+  return add(mul(-d.Lbar[o].w, nv), mul(id, sub(nb, mul(nbn, nv))));
 }
 
 // Ubar[cur] holds the own-contact part of the adjoint of U^0 (completed here with
@@ -342,7 +374,7 @@ __global__ void __launch_bounds__(kAdjThreads) k_adj_geom(StepArgs a, AdjArgs d,
   float part[kPart] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
   if (i < a.n) {
     (void)complete_ubar(a, d, i, d.Ubar[cur][i], d.ubar[0]);
-    const size_t n = a.n, KN = (size_t)a.K * n, KbN = (size_t)a.Kb * n;
+    const size_t n = a.n, KbN = (size_t)a.Kb * n;
     const float4 pi = a.pos_id[i];
     float3 X = f3(d.xbar_s[i]);
     const uint32_t cc = a.ccount[i];
@@ -352,7 +384,7 @@ __global__ void __launch_bounds__(kAdjThreads) k_adj_geom(StepArgs a, AdjArgs d,
       const uint32_t j = a.cj[o];
       const float dist = pi.w + a.pos_id[j].w - a.cn[o].w;
       const size_t ot = (size_t)d.twin[o] * n + j;
-      X = add(X, sub(pair_geom_grad(d, a, o, KN, dist), pair_geom_grad(d, a, ot, KN, dist)));
+      X = add(X, sub(pair_geom_grad(d, a, o, dist), pair_geom_grad(d, a, ot, dist)));
     }
     const float3 xi = f3(pi);
     for (uint32_t c = 0; c < nbc; ++c) {
@@ -391,7 +423,7 @@ __global__ void __launch_bounds__(kAdjThreads) k_adj_geom(StepArgs a, AdjArgs d,
     const float4 b = d.basebar[i];
     d.vbar[id] = make_float4(b.x, b.y, b.z, 0.f);
   }
-  block_partials(part, d.part + ((size_t)d.I * d.nblk + blockIdx.x) * kPart);
+  block_partials<false>(part, d.part + ((size_t)2 * d.nblk_iter + blockIdx.x) * kPart);
 }
 
 __device__ void rodrigues(float3 phi, float R[9]) {
@@ -433,7 +465,7 @@ __device__ void left_jacobian(float3 phi, float J[9]) {
     }
 }
 
-// Sums the partials in a fixed order (thread-strided over the (sweep, block) vectors in
+// Sums the partials in a fixed order (thread-strided over the blocks' vectors in
 // float, a fixed butterfly in each warp, then the warps in index order in double), and
 // thread 0 runs the tool pose chain of step k.  k is the step counter less the one saved
 // with the taped run's first checkpoint (`ctrl0`), so one captured graph serves every
@@ -446,15 +478,15 @@ __global__ void __launch_bounds__(kToolThreads) k_adj_tool(StepArgs a, AdjArgs d
   float f[16];
 #pragma unroll
   for (int q = 0; q < 16; ++q) f[q] = 0.f;
-  const uint32_t I = d.I, nb = d.nblk;
+  const uint32_t ni = d.I ? d.nblk_iter : 0u, nb = d.nblk;
 #pragma unroll 2
-  for (uint32_t t = threadIdx.x; t < I * nb; t += kToolThreads) {  // t = s * nblk + b
-    const float *p = d.part + (size_t)t * kPart;
+  for (uint32_t t = threadIdx.x; t < ni; t += kToolThreads) {
+    const float *p = d.part + (size_t)t * 2 * kPart;
 #pragma unroll
     for (int q = 0; q < kPart; ++q) f[q] += p[q];
   }
   for (uint32_t b = threadIdx.x; b < nb; b += kToolThreads) {
-    const float *g = d.part + ((size_t)I * nb + b) * kPart;
+    const float *g = d.part + ((size_t)2 * d.nblk_iter + b) * kPart;
 #pragma unroll
     for (int q = 0; q < 6; ++q) f[10 + q] += g[q];
   }
@@ -533,6 +565,15 @@ cudaError_t enqueue_copy_regions(const CopyRegions &c, cudaStream_t st) {
 
 uint32_t adjoint_blocks(uint32_t n) { return blocks(n); }
 
+// Lanes a particle of the reversed sweeps.  A reverse step (taped step and adjoint) with one
+// thread a particle, and with 8, 4 and 2 lanes: 2,000 spheres 377, 310, 360, 421 us; 16,000
+// 434, -, 418, -; 32,768 418, 482, 409, 460; 131,072 873, 1247, 962, 843; 500,000 3467,
+// 4850, 3598, 3138 (more lanes shorten the chain and add instructions).
+static uint32_t lanes_per_particle(uint32_t n) { return n <= 8192u ? 8u : (n <= 65536u ? 4u : 2u); }
+uint32_t adjoint_iter_blocks(uint32_t n) {
+  return std::max(1u, (uint32_t)(((size_t)n * lanes_per_particle(n) + kAdjThreads - 1) / kAdjThreads));
+}
+
 // The step's adjoint kernels, chained with programmatic dependent launch (every one
 // begins with pdl_enter); the first follows the body-frame kernel of the step.
 cudaError_t enqueue_adjoint_step(const StepArgs &a, const AdjArgs &d, const DevCtrl *ctrl0, uint32_t n_taped,
@@ -543,9 +584,11 @@ cudaError_t enqueue_adjoint_step(const StepArgs &a, const AdjArgs &d, const DevC
     if ((e = launch(true, k_adj_twins, g, kAdjThreads, 0, st, a, d)) != cudaSuccess) return e;
     if ((e = launch(true, k_adj_begin, g, kAdjThreads, 0, st, a, d)) != cudaSuccess) return e;
   }
+  const uint32_t lanes = lanes_per_particle(a.n);
+  const auto iter = lanes == 8u ? k_adj_iter<8> : (lanes == 4u ? k_adj_iter<4> : k_adj_iter<2>);
   int cur = 0;
   for (int s = (int)d.I - 1; s >= 0; --s) {
-    if ((e = launch(true, k_adj_iter, g, kAdjThreads, 0, st, a, d, (uint32_t)s, cur)) != cudaSuccess) return e;
+    if ((e = launch(true, iter, dim3(d.nblk_iter), kAdjThreads, 0, st, a, d, (uint32_t)s, cur)) != cudaSuccess) return e;
     cur ^= 1;
   }
   if ((e = launch(true, k_adj_geom, g, kAdjThreads, 0, st, a, d, cur)) != cudaSuccess) return e;

@@ -1400,7 +1400,7 @@ gg_status gg_tape_reserve(gg_sim *s, uint32_t n_steps, uint32_t K) {
   s->ad.allocs.clear();
   s->ad.taped = 0;
   const size_t n = s->n, I = s->ls.iters, KN = (size_t)s->K * n, KbN = (size_t)s->Kb * n;
-  const uint32_t nblk = gg::adjoint_blocks(s->n);
+  const uint32_t nblk = gg::adjoint_blocks(s->n), nblk_iter = gg::adjoint_iter_blocks(s->n);
   s->ad.state_bytes = (state_bytes(s) + 255) / 256 * 256;
   const size_t nck = (n_steps + K - 1) / K;
   const size_t slots = std::min(K, n_steps);  // steps of a segment, each with its own tape
@@ -1414,17 +1414,18 @@ gg_status gg_tape_reserve(gg_sim *s, uint32_t n_steps, uint32_t K) {
       (rc = ad_alloc(s, &s->ad.cn, slots * KN)) || (rc = ad_alloc(s, &s->ad.bj, slots * KbN)) ||
       (rc = ad_alloc(s, &s->ad.bn, slots * KbN)) || (rc = ad_alloc(s, &s->ad.bxc, slots * KbN)) ||
       (rc = ad_alloc(s, &d.twin, KN)) || (rc = ad_alloc(s, &d.Ubar[0], n)) || (rc = ad_alloc(s, &d.Ubar[1], n)) ||
-      (rc = ad_alloc(s, &d.ubar[0], 3 * KN)) || (rc = ad_alloc(s, &d.ubar[1], 3 * KN)) || (rc = ad_alloc(s, &d.Lbar, 3 * KN)) || (rc = ad_alloc(s, &d.bLbar, 3 * KbN)) ||
-      (rc = ad_alloc(s, &d.psibar, KN)) || (rc = ad_alloc(s, &d.nbar, 3 * KN)) || (rc = ad_alloc(s, &d.bpsibar, KbN)) ||
+      (rc = ad_alloc(s, &d.ubar[0], KN)) || (rc = ad_alloc(s, &d.ubar[1], KN)) || (rc = ad_alloc(s, &d.Lbar, KN)) || (rc = ad_alloc(s, &d.bLbar, 3 * KbN)) ||
+      (rc = ad_alloc(s, &d.nbar, KN)) || (rc = ad_alloc(s, &d.bpsibar, KbN)) ||
       (rc = ad_alloc(s, &d.bnbar, 3 * KbN)) || (rc = ad_alloc(s, &d.bxcbar, 3 * KbN)) ||
       (rc = ad_alloc(s, &d.basebar, n)) || (rc = ad_alloc(s, &d.xbar_s, n)) || (rc = ad_alloc(s, &d.xbar, n)) ||
-      (rc = ad_alloc(s, &d.vbar, n)) || (rc = ad_alloc(s, &d.part, (I + 1) * nblk * 10)) ||
+      (rc = ad_alloc(s, &d.vbar, n)) || (rc = ad_alloc(s, &d.part, ((size_t)2 * nblk_iter + nblk) * 10)) ||
       (rc = ad_alloc(s, &d.pose_bar, 6)) || (rc = ad_alloc(s, &d.dtwist, (size_t)n_steps * 6)) ||
       (rc = ad_alloc(s, &d.mubar, 1)))
     return rc;
   d.tp = tp;
   d.I = (uint32_t)I;
   d.nblk = nblk;
+  d.nblk_iter = nblk_iter;
   d.tool = 0xffffffffu;
   s->ad.n_steps = n_steps;
   s->ad.K = K;

@@ -484,17 +484,19 @@ struct AdjArgs {
   Tape tp;
   uint32_t I;              // sweeps per step
   uint32_t tool;           // global body index whose twists are differentiated (~0u: none)
-  uint32_t nblk;           // blocks of the per-particle adjoint kernels
+  uint32_t nblk;           // blocks of the per-particle adjoint kernels ...
+  uint32_t nblk_iter;      // ... and of the reversed sweeps
   uint32_t *twin;          // [K][n] position of contact (j -> i) in j's list
   float4 *Ubar[2];         // adjoint of U^{s+1} / U^s
-  float *ubar[2];          // [3][K][n] adjoint of each pair contact's relative velocity, by sweep parity
-  float *Lbar, *bLbar;     // [3][K][n], [3][Kb][n] adjoint of lambda^s (carried down the sweeps)
-  float *psibar, *nbar;    // [K][n], [3][K][n]
+  float4 *ubar[2];         // [K][n] adjoint of each pair contact's relative velocity, by sweep parity
+  float4 *Lbar;            // [K][n] adjoint of lambda^s (carried down the sweeps), psi-bar in w
+  float *bLbar;            // [3][Kb][n] the same of the body contacts
+  float4 *nbar;            // [K][n]
   float *bpsibar, *bnbar, *bxcbar;  // [Kb][n], [3][Kb][n], [3][Kb][n]
   float4 *basebar;         // adjoint of v + dt g
   float4 *xbar_s;          // adjoint of x_{k+1} (working copy)
   float4 *xbar, *vbar;     // id order: in dL/dx_{k+1}, dL/dv_{k+1}; out dL/dx_k, dL/dv_k
-  float *part;             // [I + 1][nblk][10] fixed-order partial sums
+  float *part;             // [nblk_iter][2][10], then [nblk][10]: fixed-order partial sums
   float *pose_bar;         // [6] adjoint of the tool pose (p, rotation), updated per step
   float *dtwist;           // [steps][6] output
   double *mubar;           // [1] dL/dmu, accumulated

@@ -76,6 +76,7 @@ cudaError_t enqueue_sort_from_keys(const StepArgs &a, cudaStream_t st);
 cudaError_t enqueue_adjoint_step(const StepArgs &a, const AdjArgs &d, const DevCtrl *ctrl0, uint32_t n_taped,
                                  cudaStream_t st);
 uint32_t adjoint_blocks(uint32_t n);
+uint32_t adjoint_iter_blocks(uint32_t n);
 // up to four regions of 32-bit words (unused ones with zero words), copied in one launch
 struct CopyRegions {
   uint32_t *dst[4];

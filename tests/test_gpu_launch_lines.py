@@ -1,5 +1,5 @@
 """Both sides of the lines at which a launch changes its shape: the depth camera's warp per
-body, the half-stencil search's thread per row, the reverse pass's kept graphs."""
+body, the half-stencil search's thread per row, the reverse pass's kept graphs and lanes."""
 import numpy as np
 import pytest
 
@@ -88,3 +88,33 @@ def test_reverse_passes_of_changing_length(gg):
         one.close()
         assert np.array_equal(got[0], want[0]) and got[1] == want[1]
     kept.close()
+
+
+@pytest.mark.parametrize("n", [65, 8192, 8193, 65536, 65537])
+def test_reverse_pass_lanes(gg, n):
+    """The reversed sweeps take 8, 4 or 2 lanes a particle by the particle count.  With the
+    scene's ids reversed every sum falls to other lanes and blocks, and the gradient is the
+    same.  float32 sums of at most 65,537 terms, in a tree of at most 512 strided terms and
+    nine levels: 1e-4 of their size."""
+    side = int(np.ceil(np.sqrt(n)))
+    g = np.stack(np.meshgrid(np.arange(side), np.arange(side), indexing="ij"), -1).reshape(-1, 2)[:n]
+    pr = np.empty((n, 4), F32)
+    pr[:, :2] = 0.0198 * (g - side // 2)
+    pr[:, 2] = 0.0099
+    pr[:, 3] = 0.01
+    seed = np.zeros((n, 3), F32)
+    seed[:, 0], seed[:, 2] = 1.0, np.where(np.arange(n) % 3 == 0, 1.0, 0.5)
+    got = []
+    for order in (np.arange(n), np.arange(n)[::-1].copy()):
+        sim = gg.Sim(np.ascontiguousarray(pr[order]), None, S.sphere_mass(pr[:, 3]),
+                     S.Params(dt=1e-4, mu=0.5, pja_iters=4, max_contacts=8))
+        sim.set_bodies([S.Body(kind=S.PLANE, lin_vel=(0.05, 0.0, 0.1))])
+        sim.set_trajectory(0, np.tile(np.array([[0.05, 0.0, 0.1, 0.0, 0.0, 0.0]], F32), (2, 1)))
+        sim.tape_reserve(2, 2)
+        sim.step_taped(0, 2)
+        g_tw, g_mu = sim.backward(np.ascontiguousarray(seed[order]))
+        sim.close()
+        got.append((np.asarray(g_tw, np.float64), float(g_mu)))
+    scale = np.abs(got[0][0]).max()
+    assert scale > 0 and np.isfinite(got[0][0]).all()
+    assert np.abs(got[0][0][:, :3] - got[1][0][:, :3]).max() <= 1e-4 * scale
