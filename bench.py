@@ -776,6 +776,8 @@ def measure(sim, sc, steps, stream, torch, flush, workload="column", readback=No
     if sweep_kernel == contact_kernels:   # detection and sweeps in one launch per step
         roofs = [roof(sweep_kernel, pja_ms + con_ms, pja_b + con_b, len(sampled)), None]
     else:
+        if sweep_kernel == "k_flow":      # reads and writes a contact's record once for all its sweeps
+            pja_b /= sc.params.pja_iters
         sweep_launches = len(sampled) * (1 if sweep_kernel in ("k_pja_fused", "k_flow") else sc.params.pja_iters)
         roofs = [roof(sweep_kernel, pja_ms, pja_b, sweep_launches),
                  roof(contact_kernels, con_ms, con_b, len(sampled))]

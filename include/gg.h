@@ -105,7 +105,7 @@ typedef struct {
   uint32_t tuning;           /* 0: the first gg_step times every launch-shape set (binning
                                 included) on a copy of the state (restored bit-exactly) and keeps
                                 the fastest; k >= 1: fixed set k (see gg_tuning_count; sets 7-9,
-                                11-12 bin by linked lists, sets 9, 10, 12 cap the sweep at 40
+                                11-12 bin by linked lists, sets 9, 10, 12 cap the sweep at 56
                                 registers, sets 11-13 find pairs over half the stencil and mirror
                                 them, sets 14-15 (sort, lists) run detection and every sweep in one
                                 cooperative launch, sets 16-18 (sort, lists, lists with the half
@@ -113,8 +113,10 @@ typedef struct {
                                 records, sets 19-20 (sort, lists) run the paper's OneLoop: every
                                 iteration walks the cells again and computes each response as it
                                 finds the contact, set 21 is set 11 with 128-thread sweep
-                                blocks, set 22 is set 18 with the 40-register sweep and no
-                                preloaded round).  Results do not depend on it. */
+                                blocks, set 22 is set 18 with the 56-register sweep and no
+                                preloaded round, sets 23-25 (sort, lists, lists with the half
+                                stencil) run every sweep in one launch that keeps the contact
+                                records on chip).  Results do not depend on it. */
   uint32_t wrench_history;   /* per-step body wrenches kept for readback; 0 -> 1 */
   uint32_t max_free_bodies;  /* free rigid bodies over all environments (beyond the paper's
                                 kinematic bodies, Sec. V two-way coupling); 0 -> none */

@@ -129,7 +129,7 @@ struct gg_sim {
     float4 *cn = nullptr, *bn = nullptr, *bxc = nullptr;
     gg::AdjArgs d{};
     // the reverse pass's graphs, one per slot and direction, kept between reverse passes of
-    // the same length and tool (capturing them took 2 of 12 ms for 20 steps)
+    // the same length and tool (20 steps and their reverse 11.7 -> 10.7 ms)
     std::vector<cudaGraphExec_t> fwd, adj;
     uint32_t graph_steps = 0, graph_tool = 0xffffffffu;
     std::vector<void *> allocs;

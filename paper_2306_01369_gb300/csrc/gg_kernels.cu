@@ -1265,8 +1265,8 @@ __device__ __forceinline__ void advance_pose(float dt, float p[3], float q[4], c
 
 // Free-box corners: +lambda on the box, -lambda on the other body, added to thread 0's v in
 // the order (box, corner, other body).  The block looks at kWrenchBodyThreads of them at a
-// time and thread 0 adds the few that count (one thread reading all of them in turn took
-// 35 us of the excavation's step).
+// time and thread 0 adds the few that count (with one thread reading all of them in
+// turn the kernel took 42.7 us of the excavation's step, now 9.7).
 constexpr int kWrenchBodyThreads = 256;
 
 __device__ __forceinline__ void add_corners(const StepArgs &a, uint32_t gb, uint32_t e, const float p[3], float v[6]) {
