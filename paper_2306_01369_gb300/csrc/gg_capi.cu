@@ -802,7 +802,7 @@ gg_status gg_create_batch(const gg_params *params, uint32_t n_envs, const uint32
   // after another (whole environments, as many as fit the shared memory of the chip)
   uint32_t *wave_off = nullptr;
   if ((rc = dalloc(s, &a.T[0], n)) || (rc = dalloc(s, &a.T[1], n)) ||
-      (rc = dalloc(s, &a.epoch, 1)) || (rc = dalloc(s, &a.farr, s->F)) || (rc = dalloc(s, &a.ftw, (size_t)s->F * 4)) ||
+      (rc = dalloc(s, &a.epoch, 1)) || (rc = dalloc(s, &a.list_sym, gg::kSymSlots * gg::kSymStride)) || (rc = dalloc(s, &a.farr, s->F)) || (rc = dalloc(s, &a.ftw, (size_t)s->F * 4)) ||
       (rc = dalloc(s, &wave_off, (size_t)n_envs + 1)))
     return bail(rc);
   a.tag_step = P.pja_iters + 2u;
@@ -855,6 +855,7 @@ gg_status gg_create_batch(const gg_params *params, uint32_t n_envs, const uint32
       (e = cudaMemset(a.key_id, 0, sizeof(uint32_t) * std::max(n, 1u))) != cudaSuccess ||
       (e = cudaMemset(a.ctrl, 0, sizeof(DevCtrl))) != cudaSuccess ||
       (e = cudaMemset(a.epoch, 0, sizeof(uint32_t))) != cudaSuccess ||
+      (e = cudaMemset(a.list_sym, 0, sizeof(uint32_t) * gg::kSymSlots * gg::kSymStride)) != cudaSuccess ||
       (e = cudaMemset(a.tile_work, 0, sizeof(uint32_t) * (((size_t)n + 31) / 32 + 4))) != cudaSuccess ||
       (e = cudaMemset(a.T[0], 0, sizeof(float4) * std::max(n, 1u))) != cudaSuccess ||
       (e = cudaMemset(a.T[1], 0, sizeof(float4) * std::max(n, 1u))) != cudaSuccess ||

@@ -34,6 +34,9 @@ constexpr uint32_t kMaxBucket = 1024;
 // Tags of the dataflow sweeps (gg_flow.cu) start over past this one.
 constexpr uint32_t kTagLimit = 0x30000000u;
 
+// Slots the lists' symmetry sum is spread over (a 32-byte sector each, a lane reads each).
+constexpr uint32_t kSymSlots = 32, kSymStride = 8;
+
 constexpr uint32_t kListEnd = 0xffffffffu;  // end of a bucket's linked list
 constexpr int kMaxK = 32;   // particle-particle capacity limit
 constexpr int kMaxKb = 8;   // particle-body capacity limit
@@ -188,6 +191,7 @@ struct StepArgs {
   uint2 *flow_r;          // place and flags, partner
   float4 *flow_b;         // body contacts: point velocity or lever arm
   uint32_t *epoch;        // tag base of the next launch
+  uint32_t *list_sym;     // [kSymSlots * kSymStride] per-step sum that is zero if the contact lists are symmetric
   uint32_t tag_step;      // tags a step takes
   uint32_t *farr;         // [F] free-body contacts updated so far in this launch
   float4 *ftw;            // [F][2][2] a free body's (v, tag), (w, -) by iteration parity

@@ -23,10 +23,11 @@
 // or barrier is involved.  Two slots by iteration parity suffice: i overwrites U^s with
 // U^{s+2} only after reading U^{s+1} of every partner, which each partner publishes only
 // after it has read U^s_i -- because contact lists are symmetric.  They are unless detection
-// cut one short (a latched capacity or bucket flag); then, and where a block's lists would
-// not fit its shared memory, the launch runs the plain sweeps with a grid barrier between
-// them, like k_pja_fused.  A wait is bounded (wait_cycles), latches kFlagTimeout and makes
-// every later wait return at once.
+// cut one short (a latched capacity or bucket flag) or a sphere is larger than the cells
+// allow (the lists' symmetry sum is not zero then); in those cases, and where a block's
+// lists would not fit its shared memory, the launch runs the plain sweeps with a grid barrier
+// between them, like k_pja_fused.  A wait is bounded (wait_cycles), latches kFlagTimeout and
+// makes every later wait return at once.
 //
 // All blocks are resident (cooperative launch, one block per SM).  A batch is swept in
 // ranges of whole environments that fit the chip, one after another with no barrier between
@@ -243,8 +244,12 @@ constexpr uint32_t kFarChunk = 1280;        // 32 x (N 16, L 16, place and flags
 constexpr uint32_t kBody = 0x10000u, kFree = 0x20000u, kNear = 0x40000u;  // flags of a far / memory record
 // references: the impulse's offset, or with kMem the record's index in memory
 constexpr uint32_t kSign = 0x80000000u, kMem = 0x40000000u;
-constexpr uint32_t kOpen = 0x20000000u;     // (while records are made) not resolved: the rest is the partner's place
+// (while records are made) not resolved: the rest is the partner's place times 16, an offset
+// that is aligned and inside the pool should a list ever name a sphere that does not name it
+constexpr uint32_t kOpen = 0x20000000u;
 constexpr uint32_t kRefBits = 0x1fffffffu;
+
+__device__ __forceinline__ uint32_t open_ref(uint32_t place) { return kOpen | place << 4; }
 
 __device__ __forceinline__ uint32_t near_at(const Block &k, uint32_t r) { return k.rec + (r >> 5) * kNearChunk + (r & 31u) * 16u; }
 __device__ __forceinline__ uint32_t far_at(const Block &k, uint32_t r) { return k.top - ((r >> 5) + 1u) * kFarChunk + (r & 31u) * 16u; }
@@ -520,7 +525,8 @@ __global__ void __launch_bounds__(kFlowThreads, 1) k_flow(const __grid_constant_
   const uint32_t G = gridDim.x - (FREE ? a.F : 0u);
   const uint32_t out0 = *a.epoch;
   // ranges that get the plain sweeps: all of them when a list may be asymmetric
-  const bool asym = (a.ctrl->status & kAsymmetric) != 0u;
+  const bool asym = (a.ctrl->status & kAsymmetric) != 0u ||
+                    __reduce_add_sync(0xffffffffu, a.list_sym[(threadIdx.x & 31u) * kSymStride]) != 0u;
   // (a phantom participant, for tests of the bounded waits: tags that nothing writes)
   const uint32_t tag0 = out0 + (a.ctrl->bar_extra ? 0x40000000u : 0u);
   Waits wt{false};
@@ -630,7 +636,7 @@ __global__ void __launch_bounds__(kFlowThreads, 1) k_flow(const __grid_constant_
           if (!GG_GUARD(a.ctrl, code < a.n)) code = i;
           const uint32_t pl = place_of(k, code, p0, p1);
           if (pl == kNone) far = kFar;
-          else at<uint32_t>(k.ref, (row + c) * 32u + lane) = kOpen | pl;
+          else at<uint32_t>(k.ref, (row + c) * 32u + lane) = open_ref(pl);
           near = pl != kNone && pl > o;
           nf += pl == kNone ? 1u : 0u;
         } else if (c < cnt) {
@@ -655,13 +661,13 @@ __global__ void __launch_bounds__(kFlowThreads, 1) k_flow(const __grid_constant_
         uint32_t code = c < npp ? at<uint32_t>(k.ref, (row + c) * 32u + lane) : 0u;   // partner
         uint32_t word = o, kc = c;                                                    // place and flags, contact of its kind
         const bool local = c < npp && (code & kOpen);
-        if (local && (code ^ kOpen) < o) continue;
+        if (local) code = (code & kRefBits) >> 4;
+        if (local && code < o) continue;
         if (c >= npp) {
           kc = c - npp;
           code = atomicAdd(&s_nb, 1u);
           word |= kBody | (FREE && a.bodies[a.bj[(size_t)kc * n + i]].is_free ? kFree : 0u);
         }
-        if (local) code ^= kOpen;
         uint32_t ref;
         if (fits) {
           const uint32_t r = local ? rn++ : rf++;
@@ -688,7 +694,7 @@ __global__ void __launch_bounds__(kFlowThreads, 1) k_flow(const __grid_constant_
       const uint32_t pc = at<uint8_t>(k.cnt, p) & 0x7fu, pr = refs_of(k, p);
 #pragma unroll 2
       for (uint32_t d = 0; d < pc; ++d)
-        if (at<uint32_t>(pr, 32u * d) == (kOpen | o)) at<uint32_t>(pr, 32u * d) = ref | kSign;
+        if (at<uint32_t>(pr, 32u * d) == open_ref(o)) at<uint32_t>(pr, 32u * d) = ref | kSign;
     };
 #pragma unroll 1
     for (uint32_t r = tid; r < nl; r += kFlowThreads) {

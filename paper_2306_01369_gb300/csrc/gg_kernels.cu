@@ -105,6 +105,7 @@ __global__ void k_key(StepArgs a) {
     a.fcount[i] = 0;
     a.farr[i] = 0;
   }
+  if (i < kSymSlots) a.list_sym[i * kSymStride] = 0;
   // the dataflow sweeps' tags start over: forget the old ones
   if (*a.epoch == 0u && i < a.n) {
     a.T[0][i].w = 0.f;
@@ -636,6 +637,28 @@ __device__ __forceinline__ void detect_particle(const StepArgs &a, uint32_t i, u
   contact_records(a, i, pi, a.vel_id[i], e, E, fid, S, a.K, npp, ovf, nbc, psi_max);
 }
 
+// A pair's entry in its two spheres' lists counts once with each sign, so the sum over all
+// lists is zero where every pair is in both.  The dataflow sweeps need that (their waits and
+// their one record for two spheres rest on it), and a search over the whole stencil does not
+// promise it: a sphere whose radius was raised above half a cell after creation
+// (gg_set_particles) walks cells that its partner does not.  (The half-stencil search writes
+// both entries itself.)
+__device__ __forceinline__ uint32_t pair_mix(uint32_t lo, uint32_t hi) {
+  uint32_t x = lo * 0x9E3779B1u + (hi ^ (hi << 13)) * 0x85EBCA6Bu;
+  x ^= x >> 15;
+  x *= 0x2C1B3C6Du;
+  return x ^ (x >> 13);
+}
+__device__ __forceinline__ void add_symmetry(const StepArgs &a, uint32_t i, const uint32_t *fid, uint32_t S, uint32_t npp) {
+  uint32_t s = 0;
+  for (uint32_t c = 0; c < npp; ++c) {
+    const uint32_t j = fid[c * S];
+    s += i < j ? pair_mix(i, j) : 0u - pair_mix(j, i);
+  }
+  s = __reduce_add_sync(0xffffffffu, s);
+  if ((threadIdx.x & 31) == 0 && s) atomicAdd(&a.list_sym[((i >> 5) % kSymSlots) * kSymStride], s);
+}
+
 template <bool LISTS>
 __global__ void __launch_bounds__(kContactsBlock, 8) k_contacts(StepArgs a) {
   pdl_enter();
@@ -644,6 +667,7 @@ __global__ void __launch_bounds__(kContactsBlock, 8) k_contacts(StepArgs a) {
   uint32_t npp = 0, nbc = 0;
   float psi_max = 0.f;
   if (i < a.n) detect_particle<LISTS>(a, i, s_fid + threadIdx.x, blockDim.x, npp, nbc, psi_max);
+  if (a.flow) add_symmetry(a, i, s_fid + threadIdx.x, blockDim.x, npp);
   contact_stats(a, i, npp, nbc, psi_max);
 }
 

@@ -152,3 +152,29 @@ def test_going_back_to_a_checkpoint(gg):
         sim.step(3)
         assert np.array_equal(first[0], sim.pos()) and np.array_equal(first[1], sim.vel())
     sim.close()
+
+
+def test_spheres_larger_than_the_cells(gg):
+    """Radii raised after creation above half a cell: a full-stencil search then lists pairs
+    for one of their spheres only (the larger one walks cells the smaller one does not), and
+    the plain sweeps run, as bit-identical as before."""
+    sc = squeezed(3000, max_contacts=32)
+    big = sc.pos_r.copy()
+    big[::7, 3] *= np.float32(1.7)
+    for k in flow_sets(gg):
+        ref = 21 if "half" in gg.tuning_flags(k) else 7
+        got = []
+        for tuning in (ref, k):
+            sim = gg.Sim.from_scene(sc, tuning=tuning)
+            sim.set_particles(big)
+            sim.step(1)
+            c = sim.contacts()
+            own = np.repeat(np.arange(sc.n), np.diff(c["pp_off"].astype(np.int64)))
+            pairs = set(zip(own.tolist(), c["pp_j"].tolist()))
+            if "half" not in gg.tuning_flags(k):
+                assert any((j, i) not in pairs for i, j in pairs)
+            got.append([sim.read(f) for f in ("POS", "VEL", "BODY_WRENCH", "CONTACT_IMPULSE")])
+            assert sim.stats()["status_flags"] == 0
+            sim.close()
+        for a, b in zip(*got):
+            assert np.array_equal(a, b), k
