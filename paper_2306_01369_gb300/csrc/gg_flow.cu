@@ -140,10 +140,13 @@ __device__ __forceinline__ void free_twist(const StepArgs &a, const DevBody &B, 
     *W = make_float3(B.w[0], B.w[1], B.w[2]);
     return;
   }
+  // published as the angular half, a fence, then the linear half with the tag: the tag is
+  // polled by loads of the size of that store (accesses of unlike size would be a race in the
+  // memory model), and a fence stands before the angular half is read
   const float4 *p = a.ftw + ((size_t)fid * 2 + (s & 1u)) * 2;
-  const uint32_t *t = reinterpret_cast<const uint32_t *>(p) + 3;
-  wait_word(a, t, tag, w);
-  const float4 v = __ldcg(p), o = __ldcg(p + 1);
+  const float4 v = wait_tagged(a, p, ld_tagged(p), tag, w);
+  __threadfence();
+  const float4 o = __ldcg(p + 1);
   *V = make_float3(v.x, v.y, v.z);
   *W = make_float3(o.x, o.y, o.z);
 }

@@ -178,3 +178,31 @@ def test_spheres_larger_than_the_cells(gg):
             sim.close()
         for a, b in zip(*got):
             assert np.array_equal(a, b), k
+
+
+def pressed_boxes(n=3000, v=(0.0, 0.0, 0.0)):
+    """Two free boxes in use: one sunk into the top of a squeezed bed, a plate pressing on its
+    corners, one with corners in a wall of the container and its side among the spheres."""
+    sc = squeezed(n)
+    mid = float(np.median(sc.pos_r[:, 2]))
+    free = dict(is_free=1, mass=0.05, inertia=(4e-6,) * 3, lin_vel=v)
+    sc.bodies = sc.bodies + [
+        S.Body(kind=S.BOX, shape=(0.02,) * 3, pos=(0.1, 0.1, 0.115), **free),
+        S.Body(kind=S.BOX, shape=(0.01, 0.02, 0.01), pos=(0.0095, 0.1, mid), **free),
+        S.Body(kind=S.BOX, shape=(0.05, 0.05, 0.01), pos=(0.1, 0.1, 0.1445), lin_vel=(0.02, 0.0, -0.1))]
+    return sc
+
+
+def test_free_bodies_in_contact(gg):
+    """Spheres, a wall and a moving plate act on two free boxes: what the boxes' blocks and
+    the spheres' exchange in every sweep, for every set."""
+    sc = pressed_boxes()
+    sim = gg.Sim.from_scene(sc, tuning=flow_sets(gg)[0])
+    sim.step(1)
+    b = sim.contacts()["bc_b"]
+    assert all((b == k).sum() >= 5 for k in (1, 2))           # spheres on both boxes
+    assert np.abs(sim.wrench()[-1, 3]).max() > 0              # and a box's corners on the plate
+    sim.close()
+    same(gg, sc, steps=4)
+    sc.params = dataclasses.replace(sc.params, pja_iters=3)
+    same(gg, sc, steps=2)
