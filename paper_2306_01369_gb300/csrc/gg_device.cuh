@@ -31,8 +31,13 @@ constexpr uint32_t kFlagBucketBound = 64u; // a bucket held more than kMaxBucket
 // and the step reports an error instead of running for minutes.
 constexpr uint32_t kMaxBucket = 1024;
 
-// Tags of the dataflow sweeps (gg_flow.cu) start over past this one.
+// Tags of the dataflow sweeps (gg_flow.cu) start over past this one (in the debug build every
+// few steps, so that its tests cross it).
+#ifdef GG_DEBUG
+constexpr uint32_t kTagLimit = 100u;
+#else
 constexpr uint32_t kTagLimit = 0x30000000u;
+#endif
 
 // Slots the lists' symmetry sum is spread over (a 32-byte sector each, a lane reads each).
 constexpr uint32_t kSymSlots = 32, kSymStride = 8;

@@ -107,9 +107,9 @@ __global__ void k_key(StepArgs a) {
   }
   if (i < kSymSlots) a.list_sym[i * kSymStride] = 0;
   // the dataflow sweeps' tags start over: forget the old ones
-  if (*a.epoch == 0u && i < a.n) {
-    a.T[0][i].w = 0.f;
-    a.T[1][i].w = 0.f;
+  if (*a.epoch == 0u) {
+    if (i < a.n) a.T[0][i].w = a.T[1][i].w = 0.f;
+    if (i < 2u * a.F) a.ftw[2u * i].w = 0.f;
   }
   if (i == 0) {
     a.ctrl->bar_count = 0;

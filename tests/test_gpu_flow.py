@@ -4,6 +4,9 @@ per-launch sweeps: bit-identical positions, velocities, wrenches and impulses at
 where tiles, blocks and ranges end, with free bodies, several particle ranges, records
 that do not fit on chip, lists cut by the contact capacity, and bounded waits."""
 import dataclasses
+import os
+import subprocess
+import sys
 import time
 
 import numpy as np
@@ -13,6 +16,8 @@ from gpu_helpers import need_gpu
 from paper_2306_01369_gb300 import scenes as S
 
 pytestmark = pytest.mark.gpu
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 
 @pytest.fixture(scope="module")
@@ -206,3 +211,47 @@ def test_free_bodies_in_contact(gg):
     same(gg, sc, steps=4)
     sc.params = dataclasses.replace(sc.params, pja_iters=3)
     same(gg, sc, steps=2)
+
+
+RESTART = r"""
+import dataclasses, sys
+import numpy as np
+sys.path[:0] = [sys.argv[1], sys.argv[1] + "/tests"]
+from paper_2306_01369_gb300 import gg
+from test_gpu_flow import flow_sets, pressed_boxes, same
+sc = pressed_boxes()
+sc.params = dataclasses.replace(sc.params, pja_iters=3, gravity=(0.0, 0.0, 0.0))
+later = pressed_boxes(v=(0.3, -0.2, 0.4)).bodies
+apart = sc.pos_r.copy()
+apart[:, :3] *= np.float32(1.5)
+for k in flow_sets(gg):
+    same(gg, pressed_boxes(), steps=30, sets=[k])     # the tags start over every five steps
+    out = []
+    for idle in (0, 20):
+        sim = gg.Sim.from_scene(sc, tuning=k)
+        if idle:        # tags 1 and 2 published, then no free body until the tags have started over
+            sim.step(1)
+            sim.set_bodies([])
+            sim.set_particles(apart, np.zeros((sc.n, 3), np.float32))
+            sim.step(idle)
+            assert sim.stats()["n_pp"] == 0
+        sim.set_bodies(later)
+        sim.set_particles(sc.pos_r, sc.vel)
+        sim.step(1)
+        out.append([sim.read(f) for f in ("POS", "VEL", "BODY_STATE", "BODY_WRENCH")])
+        sim.close()
+    assert all(np.array_equal(a, b) for a, b in zip(*out)), k
+print("equal")
+"""
+
+
+def test_tags_that_start_over():
+    """The checked build starts its tags over after a hundred: runs across that equal the
+    split sweeps, and a free body that was out of use meanwhile is not met by the twist
+    published under the same tag before."""
+    need_gpu()
+    from paper_2306_01369_gb300 import _build
+    _build.build(debug=True)
+    r = subprocess.run([sys.executable, "-c", RESTART, ROOT], capture_output=True, text=True, timeout=600,
+                       env=dict(os.environ, GG_DEBUG="1"))
+    assert r.returncode == 0 and "equal" in r.stdout, r.stderr[-3000:]
