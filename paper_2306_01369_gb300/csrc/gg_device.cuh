@@ -39,6 +39,10 @@ constexpr uint32_t kTagLimit = 100u;
 constexpr uint32_t kTagLimit = 0x30000000u;
 #endif
 
+// StepArgs.flow: the step's sweeps are the dataflow ones, after a search that writes both
+// entries of a pair, or after one whose lists are checked for symmetry.
+constexpr uint32_t kFlowRun = 1, kFlowCheck = 2;
+
 // Slots the lists' symmetry sum is spread over (a 32-byte sector each, a lane reads each).
 constexpr uint32_t kSymSlots = 32, kSymStride = 8;
 

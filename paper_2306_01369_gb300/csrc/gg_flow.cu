@@ -528,8 +528,8 @@ __global__ void __launch_bounds__(kFlowThreads, 1) k_flow(const __grid_constant_
   const uint32_t G = gridDim.x - (FREE ? a.F : 0u);
   const uint32_t out0 = *a.epoch;
   // ranges that get the plain sweeps: all of them when a list may be asymmetric
-  const bool asym = (a.ctrl->status & kAsymmetric) != 0u ||
-                    __reduce_add_sync(0xffffffffu, a.list_sym[(threadIdx.x & 31u) * kSymStride]) != 0u;
+  const uint32_t sym = a.flow == kFlowCheck ? a.list_sym[(threadIdx.x & 31u) * kSymStride] : 0u;
+  const bool asym = ((a.ctrl->status & kAsymmetric) | __reduce_add_sync(0xffffffffu, sym)) != 0u;
   // (a phantom participant, for tests of the bounded waits: tags that nothing writes)
   const uint32_t tag0 = out0 + (a.ctrl->bar_extra ? 0x40000000u : 0u);
   Waits wt{false};

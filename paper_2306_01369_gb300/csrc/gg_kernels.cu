@@ -105,7 +105,7 @@ __global__ void k_key(StepArgs a) {
     a.fcount[i] = 0;
     a.farr[i] = 0;
   }
-  if (i < kSymSlots) a.list_sym[i * kSymStride] = 0;
+  if (a.flow == kFlowCheck && i < kSymSlots) a.list_sym[i * kSymStride] = 0;
   // the dataflow sweeps' tags start over: forget the old ones
   if (*a.epoch == 0u) {
     if (i < a.n) a.T[0][i].w = a.T[1][i].w = 0.f;
@@ -667,7 +667,7 @@ __global__ void __launch_bounds__(kContactsBlock, 8) k_contacts(StepArgs a) {
   uint32_t npp = 0, nbc = 0;
   float psi_max = 0.f;
   if (i < a.n) detect_particle<LISTS>(a, i, s_fid + threadIdx.x, blockDim.x, npp, nbc, psi_max);
-  if (a.flow) add_symmetry(a, i, s_fid + threadIdx.x, blockDim.x, npp);
+  if (a.flow == kFlowCheck) add_symmetry(a, i, s_fid + threadIdx.x, blockDim.x, npp);
   contact_stats(a, i, npp, nbc, psi_max);
 }
 
@@ -1536,7 +1536,7 @@ uint32_t kernels_per_step(const StepArgs &a, const LaunchShape &ls) {
 cudaError_t enqueue_step(const StepArgs &args, const LaunchShape &ls, cudaStream_t st, cudaEvent_t *ev, const Tape *tp,
                          bool whole) {
   StepArgs a = args;
-  a.flow = (!tp && uses_flow(a, ls)) ? 1u : 0u;
+  a.flow = (!tp && uses_flow(a, ls)) ? (ls.half ? kFlowRun : kFlowCheck) : 0u;
   a.flow_fin = ls.iters & 1u;
   cudaError_t e;
   const uint32_t nbt = a.n_envs * a.maxb;
