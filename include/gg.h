@@ -443,7 +443,10 @@ GG_API uint32_t gg_tuning_flags(uint32_t k);
  * keep the fastest table size.  gg_step does this once, on its first call, when gg_params.tuning = 0; call
  * it again when the workload changes character (a bed that has settled, a tool that
  * starts digging).  A no-op when gg_params.tuning fixes the set.  Waits for `stream`;
- * allocates a state copy for the duration of the call. */
+ * allocates a state copy for the duration of the call, and the scratch of the GG_TUNE_FLOW
+ * sets, which is kept if one of them is chosen (32 bytes a sphere, and up to 87 MB: 3 MB or
+ * less for a few thousand spheres; gg_create allocates it when tuning may choose them; where
+ * there is no memory for it those sets are left out). */
 GG_API gg_status gg_autotune(gg_sim *sim, void *stream);
 
 /* Last error message of this simulation (never NULL). */

@@ -13,6 +13,7 @@
 #include <cstring>
 #include <new>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "../../include/gg.h"
@@ -97,7 +98,8 @@ struct gg_sim {
   std::vector<float *> grids; // per body slot: samples of GRID bodies
   std::vector<uint32_t> fgb;  // free-body slot -> global body index (~0u when unused)
   uint32_t F = 0, Lcap = 0;
-  std::vector<void *> allocs;
+  std::vector<void *> allocs, flow_allocs;
+  uint32_t flow_most = 0;  // spheres of the largest range of the dataflow sweeps
   StepArgs a{};
   gg::LaunchShape ls{};
   uint32_t tuning_sel = 1;
@@ -309,6 +311,68 @@ void rot_from_quat(const float *q, float *R) {
   R[8] = 1.0f - 2.0f * (xx + yy);
 }
 
+// Blocks of a dataflow launch (0: it cannot run) and their shared memory.
+gg_status flow_launch(gg_sim *s, uint32_t *grid, uint32_t *pool) {
+  int nsm = 0;
+  GG_CUDA(s, cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, s->device));
+  const int per = gg::flow_setup(s->F != 0, pool);
+  *grid = per > 0 ? (uint32_t)(per * nsm) : 0;
+  return GG_OK;
+}
+
+void flow_release(gg_sim *s) {
+  StepArgs &a = s->a;
+  for (void *p : s->flow_allocs) cudaFree(p);
+  s->flow_allocs.clear();
+  a.T[0] = a.T[1] = a.flow_n = a.flow_l = a.flow_b = nullptr;
+  a.flow_r = nullptr;
+  a.tile_work = nullptr;
+}
+
+// The scratch of the dataflow sweeps, held while a set that runs them is selected or still to
+// be tried (released by an autotuning that chose another): two tagged estimates a sphere, and per block that can get work the records that may
+// not fit on chip and the contacts with bodies.  (152 blocks of the largest size, 87 MB, were
+// held by every simulation; now 1,000 spheres hold 1 MB and 4,096 hold 5.)  Nothing to do
+// where the sweeps cannot run.
+gg_status flow_reserve(gg_sim *s, cudaStream_t st) {
+  StepArgs &a = s->a;
+  if (a.T[0] || !gg::flow_possible(a)) return GG_OK;
+  uint32_t grid = 0, pool = 0;
+  gg_status rc = flow_launch(s, &grid, &pool);
+  if (rc != GG_OK || grid <= s->F) return rc;
+  const gg::FlowScratch f = gg::flow_scratch(a, s->flow_most, grid - s->F, pool);
+  const size_t n = s->n, rec = (size_t)f.blocks * f.records, tiles = (n + 31) / 32 + 4;
+  auto take = [&](auto **ptr, size_t count) {
+    void *p = nullptr;
+    if (cudaMalloc(&p, std::max<size_t>(count, 1) * sizeof(**ptr)) != cudaSuccess) {
+      (void)cudaGetLastError();
+      return false;
+    }
+    s->flow_allocs.push_back(p);
+    *ptr = static_cast<std::remove_reference_t<decltype(*ptr)>>(p);
+    return true;
+  };
+  if (!take(&a.T[0], n) || !take(&a.T[1], n) || !take(&a.tile_work, tiles) || !take(&a.flow_n, rec) ||
+      !take(&a.flow_l, rec) || !take(&a.flow_r, rec) || !take(&a.flow_b, (size_t)f.blocks * f.bodies)) {
+    flow_release(s);
+    return fail(s, GG_ERR_OOM, "scratch of the dataflow sweeps");
+  }
+  a.flow_region = f.records;
+  a.flow_bodies = f.bodies;
+  for (float4 *t : a.T) GG_CUDA(s, cudaMemsetAsync(t, 0, n * sizeof(float4), st));  // (no tag is zero)
+  GG_CUDA(s, cudaMemsetAsync(a.tile_work, 0, tiles * sizeof(uint32_t), st));
+  GG_CUDA(s, cudaStreamSynchronize(st));
+  return GG_OK;
+}
+
+// The same for the autotuner, which leaves those sets out where there is no memory for them.
+gg_status flow_try(gg_sim *s, cudaStream_t st) {
+  const gg_status rc = flow_reserve(s, st);
+  if (rc != GG_ERR_OOM) return rc;
+  s->err.clear();
+  return GG_OK;
+}
+
 gg_status set_shape(gg_sim *s, uint32_t k) {
   gg::LaunchShape ls = kShapes[k - 1];
   ls.iters = s->p.pja_iters;
@@ -320,10 +384,8 @@ gg_status set_shape(gg_sim *s, uint32_t k) {
     ls.fused_grid = per > 0 ? (uint32_t)(per * nsm) : 0;
   }
   if (ls.flow) {
-    int nsm = 0;
-    GG_CUDA(s, cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, s->device));
-    const int per = gg::flow_setup(s->F != 0, &ls.flow_pool);
-    ls.flow_grid = per > 0 ? (uint32_t)(per * nsm) : 0;
+    gg_status rc = flow_launch(s, &ls.flow_grid, &ls.flow_pool);
+    if (rc != GG_OK) return rc;
   }
   s->ls = ls;
   s->a.lists = ls.lists;
@@ -433,8 +495,9 @@ gg_status autotune(gg_sim *s, cudaStream_t st) {
   uint32_t best_f = s->hf;
   if (tune_nh) rc = rc == GG_OK ? set_hash_factor(s, kHashFactors[0], st) : rc;
   bool first = true;
+  if (rc == GG_OK) rc = flow_try(s, st);
   for (uint32_t k = 1; rc == GG_OK && k <= kNumShapes; ++k) {
-    if (!shape_allowed(s, k)) continue;
+    if (!shape_allowed(s, k) || (kShapes[k - 1].flow && !s->a.T[0])) continue;
     if ((rc = set_shape(s, k)) != GG_OK ||
         ((kShapes[k - 1].fused_block || kShapes[k - 1].detect) && !s->ls.fused_grid))
       continue;
@@ -478,6 +541,7 @@ gg_status autotune(gg_sim *s, cudaStream_t st) {
   if (rc == GG_OK) rc = set_cell_factor(s, best_c, st);
   if (rc == GG_OK) rc = set_shape(s, best_k);
   if (rc == GG_OK && cudaStreamSynchronize(st) != cudaSuccess) rc = cuda_fail(s, cudaGetLastError(), "autotune");
+  if (rc == GG_OK && !kShapes[best_k - 1].flow) flow_release(s);
   if (e0) cudaEventDestroy(e0);
   if (e1) cudaEventDestroy(e1);
   cudaFree(saved);
@@ -626,6 +690,7 @@ void gg_destroy(gg_sim *sim) {
     if (ev) cudaEventDestroy(ev);
   if (sim->cap) cudaStreamDestroy(sim->cap);
   for (void *p : sim->allocs) cudaFree(p);
+  for (void *p : sim->flow_allocs) cudaFree(p);
   for (void *p : sim->ad.allocs) cudaFree(p);
   for (float *t : sim->traj)
     if (t) cudaFree(t);
@@ -798,11 +863,11 @@ gg_status gg_create_batch(const gg_params *params, uint32_t n_envs, const uint32
   if ((rc = dalloc(s, &a.head, s->nh_cap)) || (rc = dalloc(s, &a.next, n)) || (rc = dalloc(s, &a.pcnt, n)) ||
       (rc = dalloc(s, &a.pscr, (size_t)2 * s->K * n)))
     return bail(rc);
-  // dataflow sweeps: tagged estimates, record scratch, and the particle ranges they take one
-  // after another (whole environments, as many as fit the shared memory of the chip)
+  // dataflow sweeps: the particle ranges they take one after another (whole environments, as
+  // many as fit the shared memory of the chip); their scratch comes with flow_reserve
   uint32_t *wave_off = nullptr;
-  if ((rc = dalloc(s, &a.T[0], n)) || (rc = dalloc(s, &a.T[1], n)) ||
-      (rc = dalloc(s, &a.epoch, 1)) || (rc = dalloc(s, &a.list_sym, gg::kSymSlots * gg::kSymStride)) || (rc = dalloc(s, &a.farr, s->F)) || (rc = dalloc(s, &a.ftw, (size_t)s->F * 4)) ||
+  if ((rc = dalloc(s, &a.epoch, 1)) || (rc = dalloc(s, &a.list_sym, gg::kSymSlots * gg::kSymStride)) ||
+      (rc = dalloc(s, &a.farr, s->F)) || (rc = dalloc(s, &a.ftw, (size_t)s->F * 4)) ||
       (rc = dalloc(s, &wave_off, (size_t)n_envs + 1)))
     return bail(rc);
   a.tag_step = P.pja_iters + 2u;
@@ -813,13 +878,7 @@ gg_status gg_create_batch(const gg_params *params, uint32_t n_envs, const uint32
   }
   waves.push_back(n);
   a.n_waves = (uint32_t)waves.size() - 1u;
-  int nsm = 0;
-  if ((cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, s->device)) != cudaSuccess || nsm < 1) nsm = 1;
-  a.flow_region = gg::kFlowRecords;
-  const size_t rec = (size_t)nsm * a.flow_region;
-  if ((rc = dalloc(s, &a.tile_work, ((size_t)n + 31) / 32 + 4)) || (rc = dalloc(s, &a.flow_n, rec)) ||
-      (rc = dalloc(s, &a.flow_l, rec)) || (rc = dalloc(s, &a.flow_r, rec)) || (rc = dalloc(s, &a.flow_b, rec)))
-    return bail(rc);
+  for (uint32_t w = 0; w < a.n_waves; ++w) s->flow_most = std::max(s->flow_most, waves[w + 1] - waves[w]);
   a.wave_off = wave_off;
   a.F = s->F;
   a.Lcap = s->Lcap;
@@ -856,9 +915,6 @@ gg_status gg_create_batch(const gg_params *params, uint32_t n_envs, const uint32
       (e = cudaMemset(a.ctrl, 0, sizeof(DevCtrl))) != cudaSuccess ||
       (e = cudaMemset(a.epoch, 0, sizeof(uint32_t))) != cudaSuccess ||
       (e = cudaMemset(a.list_sym, 0, sizeof(uint32_t) * gg::kSymSlots * gg::kSymStride)) != cudaSuccess ||
-      (e = cudaMemset(a.tile_work, 0, sizeof(uint32_t) * (((size_t)n + 31) / 32 + 4))) != cudaSuccess ||
-      (e = cudaMemset(a.T[0], 0, sizeof(float4) * std::max(n, 1u))) != cudaSuccess ||
-      (e = cudaMemset(a.T[1], 0, sizeof(float4) * std::max(n, 1u))) != cudaSuccess ||
       (e = cudaMemset(a.ftw, 0, sizeof(float4) * std::max(4 * s->F, 1u))) != cudaSuccess ||
       (e = cudaMemset(a.ncb, 0, sizeof(uint32_t) * nbt)) != cudaSuccess ||
       (e = cudaMemset(a.fgb, 0xff, sizeof(uint32_t) * std::max(s->F, 1u))) != cudaSuccess ||
@@ -874,6 +930,11 @@ gg_status gg_create_batch(const gg_params *params, uint32_t n_envs, const uint32
       return bail(cuda_fail(s, e, "initialising the control word"));
   }
   s->tuning_sel = P.tuning ? P.tuning : (P.binning == 2 ? 7u : 1u);
+  if (!P.tuning)
+    rc = flow_try(s, nullptr);
+  else if (kShapes[P.tuning - 1].flow)
+    rc = flow_reserve(s, nullptr);
+  if (rc != GG_OK) return bail(rc);
   if (!shape_allowed(s, s->tuning_sel)) return bail(fail(s, GG_ERR_INVALID_ARG, "tuning set and binning disagree"));
   if ((rc = set_shape(s, s->tuning_sel)) != GG_OK) return bail(rc);
   *out = s;

@@ -194,11 +194,12 @@ struct StepArgs {
   const uint32_t *wave_off;
   float4 *T[2];           // tagged velocity estimates: x, y, z, tag (launch epoch + iteration)
   uint32_t *tile_work;    // [ceil(n / 32)] per 32 spheres: their contacts this step, the most of one << 16
-  uint32_t flow_region;   // record scratch of one block (entries of the arrays below): what does not fit on chip
+  uint32_t flow_region;   // record scratch of one block (entries of flow_n, _l, _r): what does not fit on chip
+  uint32_t flow_bodies;   // the same of flow_b
   float4 *flow_n;         // [blocks][flow_region] normal, bias
   float4 *flow_l;         // impulse, effective mass
   uint2 *flow_r;          // place and flags, partner
-  float4 *flow_b;         // body contacts: point velocity or lever arm
+  float4 *flow_b;         // [blocks][flow_bodies] body contacts: point velocity or lever arm
   uint32_t *epoch;        // tag base of the next launch
   uint32_t *list_sym;     // [kSymSlots * kSymStride] per-step sum that is zero if the contact lists are symmetric
   uint32_t tag_step;      // tags a step takes

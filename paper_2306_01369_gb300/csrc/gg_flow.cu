@@ -259,6 +259,7 @@ __device__ __forceinline__ uint32_t far_at(const Block &k, uint32_t r) { return 
 __device__ __forceinline__ uint32_t near_word(const Block &k, uint32_t r) { return k.rec + (r >> 5) * kNearChunk + 1024u + (r & 31u) * 4u; }
 __device__ __forceinline__ uint32_t far_word(const Block &k, uint32_t r) { return k.top - ((r >> 5) + 1u) * kFarChunk + 1024u + (r & 31u) * 4u; }
 __device__ __forceinline__ size_t scratch(const StepArgs &a) { return (size_t)blockIdx.x * a.flow_region; }
+__device__ __forceinline__ size_t body_scratch(const StepArgs &a) { return (size_t)blockIdx.x * a.flow_bodies; }
 
 __device__ __forceinline__ uint32_t place_id(uint32_t o) { return at<uint32_t>(0, o >> 5) * 32u + (o & 31u); }
 
@@ -294,7 +295,7 @@ __device__ __forceinline__ float4 update(const StepArgs &a, float4 nn, float4 la
 
 // The partner's estimate of a far record, asked for (`v`) and then waited for.
 __device__ __forceinline__ float4 ask(const StepArgs &a, uint32_t of, uint32_t id, const Sweep &w) {
-  if (of & kBody) return a.flow_b[scratch(a) + id];
+  if (of & kBody) return a.flow_b[body_scratch(a) + id];
   return ld_tagged((w.s ? a.T[w.s & 1u] : a.U[0]) + id);
 }
 template <bool FREE>
@@ -309,7 +310,7 @@ __device__ __forceinline__ float4 answer(const StepArgs &a, uint32_t of, uint32_
 }
 // A free body's impulse goes to the body's block.
 __device__ __forceinline__ void give(const StepArgs &a, uint32_t of, uint32_t id, float4 l) {
-  const uint32_t gbk = __float_as_uint(a.flow_b[scratch(a) + id].w);
+  const uint32_t gbk = __float_as_uint(a.flow_b[body_scratch(a) + id].w);
   hand_over(a, a.bodies[gbk >> 3].fid, (size_t)(gbk & 7u) * a.n + place_id(of & 0xffffu), (size_t)a.Kb * a.n,
             make_float3(l.x, l.y, l.z));
 }
@@ -464,7 +465,7 @@ __device__ __forceinline__ void fill_record(const StepArgs &a, const Block &k, u
       const float3 ub = point_velocity(make_float3(B.v[0], B.v[1], B.v[2]), make_float3(B.w[0], B.w[1], B.w[2]), rx, ry, rz);
       rb = make_float4(ub.x, ub.y, ub.z, 0.f);
     }
-    a.flow_b[scratch(a) + code] = rb;
+    a.flow_b[body_scratch(a) + code] = rb;
   }
   *N = make_float4(nn.x, nn.y, nn.z, a.ab * nn.w);
   *L = make_float4(0.f, 0.f, 0.f, 1.0f / (uw + ow));
@@ -493,8 +494,9 @@ struct Share {
   uint32_t own;        // ... and their cost
   uint32_t lo, hi;     // the block's window of the cost prefix
 };
-__device__ __forceinline__ uint32_t tile_cost(uint32_t v) {
-  return v ? max((v & 0xffffu) + kTileWeight, (4u + 2u + 32u + 512u + 128u * (v >> 16)) / kBytesPerCost + 1u) : 0u;
+__host__ __device__ __forceinline__ uint32_t tile_cost(uint32_t v) {
+  const uint32_t c = (v & 0xffffu) + kTileWeight, b = (4u + 2u + 32u + 512u + 128u * (v >> 16)) / kBytesPerCost + 1u;
+  return v ? (c > b ? c : b) : 0u;
 }
 
 // f(tile, tiles with contacts before, its count word) for the thread's tiles that are in
@@ -762,6 +764,21 @@ int flow_setup(bool free, uint32_t *pool) {
   const int per = free ? flow_setup_for<true>(pool) : flow_setup_for<false>(pool);
   if (!per) (void)cudaGetLastError();
   return per;
+}
+
+// A block's share costs at most W / Gw + one tile (W the range's cost, Gw = min(grid, W /
+// kMinWork) the blocks that share it); its lists take at most kBytesPerCost bytes per cost
+// and it has at most as many records as its cost, 40 bytes each and two chunks for rounding.
+FlowScratch flow_scratch(const StepArgs &a, uint32_t most, uint32_t grid, uint32_t pool) {
+  const uint64_t per = a.K + a.Kb, tile = tile_cost((uint32_t)(32u * per | per << 16));
+  const uint64_t g = std::max(1u, grid), W = ((uint64_t)most / 32u + 2u) * tile;
+  const uint64_t share = std::max(std::min<uint64_t>(W, 2u * kMinWork - 1u), W / g) + tile;
+  const bool on_chip = share * (kBytesPerCost + 40u) + 256u + kNearChunk + kFarChunk <= pool;
+  FlowScratch f;
+  f.blocks = (uint32_t)std::min(g, std::max<uint64_t>(1u, W / kMinWork));
+  f.records = on_chip ? 0u : (uint32_t)std::min<uint64_t>(share, kFlowRecords);
+  f.bodies = (uint32_t)std::min({share, (uint64_t)kFlowRecords, (uint64_t)most * a.Kb});
+  return f;
 }
 
 cudaError_t enqueue_flow(const StepArgs &a, const LaunchShape &ls, cudaStream_t st) {

@@ -47,11 +47,21 @@ struct LaunchShape {
 // Free bodies the dataflow sweeps take: each holds a block (an SM) of its own for the
 // whole launch, so more than a few would cost more than the sweeps gain.
 constexpr uint32_t kFlowMaxFree = 8;
-inline bool uses_flow(const StepArgs &a, const LaunchShape &ls) {
-  return ls.flow && ls.flow_grid > a.F && a.n < (1u << 29) && a.n && !a.lit && a.F <= kFlowMaxFree && (!a.F || a.n_waves == 1) && a.n_waves <= 1024u;
-}
-constexpr uint32_t kFlowRecords = 10240;      // record scratch of one block, for what does not fit on chip
 constexpr uint32_t kFlowMaxWaves = 1024;     // particle ranges of one launch
+inline bool flow_possible(const StepArgs &a) {
+  return a.n && a.n < (1u << 29) && !a.lit && a.F <= kFlowMaxFree && (!a.F || a.n_waves == 1) && a.n_waves <= kFlowMaxWaves;
+}
+inline bool uses_flow(const StepArgs &a, const LaunchShape &ls) {
+  return ls.flow && ls.flow_grid > a.F && a.T[0] && flow_possible(a);
+}
+constexpr uint32_t kFlowRecords = 10240;      // most record scratch of one block, for what does not fit on chip
+// Scratch the launch can need, whatever the spheres do: blocks that get work, records of one
+// that may not fit on chip (0: all fit) and contacts with bodies of one; `most`: spheres of
+// the largest particle range.
+struct FlowScratch {
+  uint32_t blocks, records, bodies;
+};
+FlowScratch flow_scratch(const StepArgs &a, uint32_t most, uint32_t grid, uint32_t pool);
 int flow_setup(bool free, uint32_t *pool);  // resident blocks per SM, shared memory per block
 cudaError_t enqueue_flow(const StepArgs &a, const LaunchShape &ls, cudaStream_t st);
 int fused_pja_blocks_per_sm(int block);

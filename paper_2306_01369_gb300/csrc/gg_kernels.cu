@@ -107,7 +107,7 @@ __global__ void k_key(StepArgs a) {
   }
   if (a.flow == kFlowCheck && i < kSymSlots) a.list_sym[i * kSymStride] = 0;
   // the dataflow sweeps' tags start over: forget the old ones
-  if (*a.epoch == 0u) {
+  if (*a.epoch == 0u && a.T[0]) {
     if (i < a.n) a.T[0][i].w = a.T[1][i].w = 0.f;
     if (i < 2u * a.F) a.ftw[2u * i].w = 0.f;
   }
@@ -425,9 +425,11 @@ struct Stats {
 __device__ __forceinline__ Stats warp_stats(const StepArgs &a, uint32_t i, uint32_t npp, uint32_t nbc, float psi_max) {
   constexpr uint32_t kAll = 0xffffffffu;
   const uint32_t sum = __reduce_add_sync(kAll, npp | nbc << 16);  // (32 times a count below 256 each)
-  const uint32_t m_all = __reduce_max_sync(kAll, npp + nbc);
-  if ((threadIdx.x & 31) == 0 && i < a.n)
-    a.tile_work[i >> 5] = ((sum & 0xffffu) + (sum >> 16)) | m_all << 16;  // (a warp's spheres are 32 consecutive ones)
+  if (a.flow) {
+    const uint32_t m_all = __reduce_max_sync(kAll, npp + nbc);
+    if ((threadIdx.x & 31) == 0 && i < a.n)
+      a.tile_work[i >> 5] = ((sum & 0xffffu) + (sum >> 16)) | m_all << 16;  // (a warp's spheres are 32 consecutive ones)
+  }
   return {sum & 0xffffu, sum >> 16, (uint32_t)__popc(__ballot_sync(kAll, npp + nbc > 0)), __reduce_max_sync(kAll, npp),
           __reduce_max_sync(kAll, nbc), __reduce_max_sync(kAll, __float_as_uint(psi_max))};
 }

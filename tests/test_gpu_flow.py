@@ -255,3 +255,37 @@ def test_tags_that_start_over():
     r = subprocess.run([sys.executable, "-c", RESTART, ROOT], capture_output=True, text=True, timeout=600,
                        env=dict(os.environ, GG_DEBUG="1"))
     assert r.returncode == 0 and "equal" in r.stdout, r.stderr[-3000:]
+
+
+@pytest.mark.parametrize("n", [700, 3000, 20000])
+def test_crowded_clouds_on_little_scratch(gg, n):
+    """The scratch is sized by what the capacities allow: none for records where a block's
+    share fits on chip whatever the contacts, some at 20,000 spheres."""
+    pr, vel = S.random_cloud(n, 6, box=0.135 * (n / 90000) ** (1 / 3), vel_scale=0.05)
+    sc = S.Scene("cloud", pr, vel, S.sphere_mass(pr[:, 3]), [S.Body(kind=S.PLANE, pos=(0.0, 0.0, 0.0))],
+                 S.Params(dt=1e-5, max_contacts=32), 4)
+    same(gg, sc, steps=1)
+
+
+def test_memory_of_small_simulations(gg):
+    """A simulation whose set never runs the dataflow sweeps holds none of their scratch, and
+    a small one little (152 blocks' worth would be 87 MB): 32 bytes a sphere, and at 4,096
+    spheres 16 bytes for each of 131 blocks' at most 1,279 + 656 contacts with bodies, a few
+    MB, with the driver's 2 MB granularity for each of the seven buffers."""
+    torch = need_gpu()
+    sc = squeezed(4096)
+
+    def held(**kw):
+        before = torch.cuda.mem_get_info()[0]
+        sims = [gg.Sim.from_scene(sc, **kw) for _ in range(8)]
+        after = torch.cuda.mem_get_info()[0]
+        for s in sims:
+            s.close()
+        return (before - after) / 8e6
+    gg.Sim.from_scene(sc).close()                 # (the context's own allocations)
+    plain, flow = held(tuning=7), held(tuning=flow_sets(gg)[1])
+    lit = dataclasses.replace(sc.params, pja_weight=1)
+    sc.params, params = lit, sc.params
+    off = held(tuning=flow_sets(gg)[1])
+    sc.params = params
+    assert flow - plain < 22 and off - plain < 2, (plain, flow, off)
