@@ -311,12 +311,13 @@ void rot_from_quat(const float *q, float *R) {
   R[8] = 1.0f - 2.0f * (xx + yy);
 }
 
-// Blocks of a dataflow launch (0: it cannot run) and their shared memory.
+// Blocks of a dataflow launch (0: it cannot run) and their shared memory: a cooperative
+// launch waits for that many empty SMs, so no more than a crowded range can use.
 gg_status flow_launch(gg_sim *s, uint32_t *grid, uint32_t *pool) {
   int nsm = 0;
   GG_CUDA(s, cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, s->device));
   const int per = gg::flow_setup(s->F != 0, pool);
-  *grid = per > 0 ? (uint32_t)(per * nsm) : 0;
+  *grid = per > 0 ? std::min((uint32_t)(per * nsm), s->F + gg::flow_blocks(s->flow_most)) : 0;
   return GG_OK;
 }
 

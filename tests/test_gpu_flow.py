@@ -289,3 +289,27 @@ def test_memory_of_small_simulations(gg):
     off = held(tuning=flow_sets(gg)[1])
     sc.params = params
     assert flow - plain < 22 and off - plain < 2, (plain, flow, off)
+
+
+def test_two_simulations_in_two_streams(gg):
+    """Small simulations claim the blocks they can use, so two run side by side: each as on
+    its own, the waits of neither held up by the other."""
+    torch = need_gpu()
+    k = flow_sets(gg)[-1]
+    scenes = [squeezed(4096), squeezed(3000, seed=12)]
+    want = []
+    for sc in scenes:
+        sim = gg.Sim.from_scene(sc, tuning=k)
+        sim.step(60)
+        want.append((sim.pos(), sim.vel()))
+        sim.close()
+    sims = [gg.Sim.from_scene(sc, tuning=k) for sc in scenes]
+    streams = [torch.cuda.Stream() for _ in sims]
+    torch.cuda.synchronize()
+    for _ in range(20):
+        for sim, st in zip(sims, streams):
+            sim.step(3, stream=st.cuda_stream)
+    torch.cuda.synchronize()
+    for sim, (x, v) in zip(sims, want):
+        assert np.array_equal(sim.pos(), x) and np.array_equal(sim.vel(), v)
+        sim.close()
