@@ -11,10 +11,11 @@
 //
 // An image is a chain of short kernels, so they are chained with programmatic dependent
 // launch and each does as little as it can: the spheres are taken last id first (beds are
-// laid down bottom up, so what a camera above sees comes early) and a value goes to its
-// pixel's atomic only if it beats what is already there; a ray stops being traced where the
-// spheres already block it.  A 72 x 36 height map and a 36 x 36 depth image of 262,144
-// spheres: 60.7 -> 41.0 us, most of it k_depth.
+// laid down bottom up, so what a camera above sees comes early), and a ray stops being traced
+// where the spheres already block it.  A look at a pixel before its atomic does not pay: the
+// atomics are not waited for, the look is, at every pixel of a sphere's loop (height map of
+// 4,000 spheres at 640 x 480 178 us without and 775 with it, of 16,000 at 160 x 96 14.5 and
+// 34.3, of 262,144 at 72 x 36 9.7 and 10.4; only 600,000 at 640 x 480 gained, 79 and 70).
 #include <algorithm>
 
 #include <cuda_runtime.h>
@@ -66,8 +67,7 @@ __global__ void k_splat_height(StepArgs a, uint32_t off, uint32_t n, RenderArgs 
       const float d2 = __fadd_rn(__fmul_rn(dx, dx), __fmul_rn(dy, dy));
       if (!(d2 <= r2)) continue;
       const float h = __fadd_rn(p.z, __fsqrt_rn(__fsub_rn(r2, d2)));
-      uint32_t *px_at = &img[(size_t)v * c.W + u];
-      if (ordered(h) > __ldcg(px_at)) atomicMax(px_at, ordered(h));  // (a pixel only grows)
+      atomicMax(&img[(size_t)v * c.W + u], ordered(h));  // (nothing waits for it; a look first made its loop wait)
     }
   }
 }
@@ -154,22 +154,73 @@ __device__ __forceinline__ void splat_depth(const StepArgs &a, uint32_t off, uin
       if (!(disc >= 0.0f)) continue;
       const float t0 = __fsub_rn(b, __fsqrt_rn(disc));
       if (!(t0 >= c.near && t0 <= c.far)) continue;
-      uint32_t *px_at = &img[(size_t)v * c.W + u];
-      if (__float_as_uint(t0) < __ldcg(px_at)) atomicMin(px_at, __float_as_uint(t0));  // t0 > 0: bits order as floats
+      atomicMin(&img[(size_t)v * c.W + u], __float_as_uint(t0));  // t0 > 0: bits order as floats
     }
 }
 
 // The spheres' and the bodies' depths of a pixel meet in its atomic, so both are made in one
-// launch: the first blocks trace 32 pixels each with a warp per body, so that a step's bodies
-// are evaluated side by side and without divergence between their kinds, and the blocks after
-// them splat the spheres meanwhile.  A traced ray is a chain of up to c.steps evaluations:
-// that chain is what the launch takes.  Every warp of a tracing block keeps the state of all
-// its pixels, so a step has one barrier (the distances are double-buffered); a ray ends where
-// the spheres already block it (their depth is looked up every fourth step: it only falls,
-// and a later hit would lie behind it).  One thread per pixel, the bodies in turn, after the
-// splat: 10.9 us for 262,144 spheres, then 33.8 us for 36 x 36 rays and two bodies; now 29.2
-// together.
+// launch: the first blocks trace, the blocks after them splat the spheres meanwhile.  A traced
+// ray is a chain of up to c.steps evaluations: that chain is what the launch takes, until the
+// image fills the chip.  A ray ends where the spheres already block it (their depth is looked
+// up every fourth step: it only falls, and a later hit would lie behind it).  Two forms, equal
+// to the bit:
+//  - k_depth: a block traces 32 pixels with a warp per body, so that a step's bodies are
+//    evaluated side by side and without divergence between their kinds.  Every warp keeps the
+//    state of all the block's pixels, so a step has one barrier (the distances are
+//    double-buffered).  Shortens the chain: 36 x 36 rays past two bodies and 262,144 spheres
+//    26.8 us, 32.9 in the other form; past eight 49 and 170.
+//  - k_depth_pixels: a thread per pixel, the bodies in turn, no barrier.  Less work in all, so
+//    it is the form of images that fill the chip: 640 x 480 past two bodies and 600,000 spheres
+//    161 us, 255 in the other form.
+// (As launches of their own, splat then trace: 47.3, 178 and 215 us.)
 constexpr uint32_t kTraceBodies = 32;  // as many as the mask has bits
+
+// Pixels up to which the bodies get a warp each.  The two forms cross between these sizes (us
+// of the whole image, k_depth and k_depth_pixels): two bodies 320 x 200 (70-72, 74-78) and 512
+// x 384 (91-119, 86-92), three 400 x 300 (45, 46), four to eight 640 x 480 (111-223, 140-273)
+// and 1280 x 720 (253-572, 212-404), sixteen 640 x 480 (568, 591), 32 at 512 x 384 (1129, 1120).
+// One body has nothing to share out.
+__host__ __forceinline__ uint32_t warp_pixels(uint32_t bodies) {
+  return bodies < 2u ? 0u : (bodies < 4u ? 100000u : std::min(400000u, 5500000u / bodies));
+}
+
+__device__ __forceinline__ float nearest_body(const StepArgs &a, uint32_t gb0, uint32_t nb, uint32_t mask, float3 x, float eps) {
+  float fmin = __int_as_float(0x7f800000);
+  for (uint32_t b = 0; b < nb; ++b) {
+    if (!((mask >> b) & 1u)) continue;
+    const DevBody &B = a.bodies[gb0 + b];
+    fmin = fminf(fmin, march_sdf(B, world_to_body(B, x), eps));
+  }
+  return fmin;
+}
+
+constexpr int kDepthThreads = 128;
+__global__ void __launch_bounds__(kDepthThreads) k_depth_pixels(StepArgs a, uint32_t off, uint32_t n, uint32_t gb0, uint32_t nb,
+                                                                uint32_t tblocks, RenderArgs c, uint32_t *img) {
+  pdl_enter();
+  if (blockIdx.x >= tblocks) {
+    const uint32_t i = (blockIdx.x - tblocks) * blockDim.x + threadIdx.x;
+    if (i < n) splat_depth(a, off, n, c, i, img);
+    return;
+  }
+  const uint32_t p = blockIdx.x * blockDim.x + threadIdx.x;
+  if (p >= c.W * c.H) return;
+  const float4 d = c.rays[p];
+  float t = c.near, seen = __int_as_float(0x7f800000);
+  for (uint32_t k = 0; k < c.steps; ++k) {
+    const float block_at = seen;
+    if ((k & 3u) == 0u) seen = __uint_as_float(__ldcg(&img[p]));
+    const float3 x = make_float3(__fadd_rn(c.o[0], __fmul_rn(t, d.x)), __fadd_rn(c.o[1], __fmul_rn(t, d.y)),
+                                 __fadd_rn(c.o[2], __fmul_rn(t, d.z)));
+    const float fmin = nearest_body(a, gb0, nb, c.mask, x, c.eps);
+    if (fmin < c.eps) {
+      atomicMin(&img[p], __float_as_uint(t));  // t >= near > 0
+      return;
+    }
+    t = __fadd_rn(t, fmin);
+    if (!(t <= c.far) || t >= block_at) return;
+  }
+}
 
 __global__ void __launch_bounds__(32 * kTraceBodies) k_depth(StepArgs a, uint32_t off, uint32_t n, uint32_t gb0, uint32_t nb,
                                                              uint32_t tblocks, RenderArgs c, uint32_t *img) {
@@ -245,10 +296,13 @@ cudaError_t enqueue_render(const StepArgs &a, uint32_t env_off, uint32_t env_n, 
     GG_CHAIN(k_finish_height, np, 256, (const uint32_t *)img, np, c.empty, out);
   } else {
     GG_CHAIN(k_begin_depth, np, 128, c, img);
-    const uint32_t nt = std::min(nb, kTraceBodies), tblocks = nt && c.mask ? cdiv(np, 32) : 0u;
-    const unsigned threads = 32u * std::max(4u, nt);
+    const uint32_t nt = std::min(nb, kTraceBodies);
+    // (of two bodies' four warps two only wait, but 64-thread blocks took 77 us where these take 70)
+    const bool warps = np <= warp_pixels(nt);
+    const unsigned threads = warps ? 32u * std::max(4u, nt) : (unsigned)kDepthThreads;
+    const uint32_t tblocks = nt && c.mask ? cdiv(np, warps ? 32u : threads) : 0u;
     if (tblocks || env_n) {
-      e = launch(true, k_depth, dim3(tblocks + (env_n ? cdiv(env_n, threads) : 0u)), threads, 0, st, a, env_off, env_n, gb0,
+      e = launch(true, warps ? k_depth : k_depth_pixels, dim3(tblocks + (env_n ? cdiv(env_n, threads) : 0u)), threads, 0, st, a, env_off, env_n, gb0,
                  nt, tblocks, c, img);
       if (e != cudaSuccess) return e;
     }

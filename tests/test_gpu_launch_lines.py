@@ -118,3 +118,28 @@ def test_reverse_pass_lanes(gg, n):
     scale = np.abs(got[0][0]).max()
     assert scale > 0 and np.isfinite(got[0][0]).all()
     assert np.abs(got[0][0][:, :3] - got[1][0][:, :3]).max() <= 1e-4 * scale
+
+
+@pytest.mark.parametrize("nb,w,h", [(1, 40, 30), (2, 400, 250), (2, 400, 251), (3, 317, 316), (4, 800, 500), (4, 800, 501),
+                                    (32, 400, 429), (32, 400, 430)])
+def test_traced_images_of_either_form(gg, orc, nb, w, h):
+    """Both sides of the pixel counts up to which a ray's bodies get a warp each: the oracle's
+    tracing to the bit, and with spheres in front the nearer of the two depths."""
+    rng = np.random.default_rng(nb)
+    bodies = [S.Body(kind=S.PLANE, pos=(0.0, 0.0, -0.3))]
+    for k in range(1, nb):
+        pos, rv = rng.uniform(-0.3, 0.3, 3), tuple(rng.uniform(-1.0, 1.0, 3))
+        bodies.append(S.Body(kind=S.BOX, shape=tuple(rng.uniform(0.02, 0.06, 3)), pos=tuple(pos),
+                             quat=S._quat_from_rotvec(rv)))
+    cam = S.Camera(kind=S.DEPTH_CAMERA, width=w, height=h, pos=(0.0, 0.0, 0.8), quat=S._quat_from_rotvec((np.pi, 0.0, 0.0)),
+                   fov_y=0.9, near=0.01, far=1.5, march_steps=24, march_eps=1e-4)
+    pr = np.concatenate([rng.uniform(-0.3, 0.3, (200, 3)), rng.uniform(0.005, 0.03, (200, 1))], 1).astype(F32)
+    out = []
+    for p, nbodies in ((pr[:0], nb), (pr, 0), (pr, nb)):
+        sim = gg.Sim(p, np.zeros((len(p), 3), F32), S.sphere_mass(p[:, 3]), S.Params(), max_bodies=nb)
+        sim.set_bodies(bodies[:nbodies])
+        out.append(sim.render(cam))
+        sim.close()
+    assert np.array_equal(out[0], orc.render(cam, np.zeros((0, 3)), np.zeros(0), bodies).astype(F32))
+    assert np.array_equal(out[2], np.minimum(out[0], out[1]))
+    assert (out[1] < out[0]).any() and (out[0] < out[1]).any()
