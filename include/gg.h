@@ -446,7 +446,9 @@ GG_API uint32_t gg_tuning_flags(uint32_t k);
  * allocates a state copy for the duration of the call, and the scratch of the GG_TUNE_FLOW
  * sets, which is kept if one of them is chosen (32 bytes a sphere, and up to 87 MB: 3 MB or
  * less for a few thousand spheres; gg_create allocates it when tuning may choose them; where
- * there is no memory for it those sets are left out). */
+ * there is no memory for it those sets are left out).  Those sets hold a step's records on
+ * chip; when most spheres no longer fit, and one of them was chosen here, a later step goes
+ * over to the fastest of the other sets (gg_tuning_selected then names that one). */
 GG_API gg_status gg_autotune(gg_sim *sim, void *stream);
 
 /* Last error message of this simulation (never NULL). */

@@ -203,6 +203,7 @@ struct StepArgs {
   uint32_t *epoch;        // tag base of the next launch
   uint32_t *list_sym;     // [kSymSlots * kSymStride] per-step sum that is zero if the contact lists are symmetric
   uint32_t tag_step;      // tags a step takes
+  uint32_t *flow_told;    // pinned host word (or null): set when most spheres get the plain sweeps
   uint32_t *farr;         // [F] free-body contacts updated so far in this launch
   float4 *ftw;            // [F][2][2] a free body's (v, tag), (w, -) by iteration parity
   // free rigid bodies

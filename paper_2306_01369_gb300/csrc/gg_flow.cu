@@ -26,7 +26,10 @@
 // cut one short (a latched capacity or bucket flag) or a sphere is larger than the cells
 // allow (the lists' symmetry sum is not zero then); in those cases, and where a block's
 // lists would not fit its shared memory, the launch runs the plain sweeps with a grid barrier
-// between them, like k_pja_fused.  A wait is bounded (wait_cycles), latches kFlagTimeout and
+// between them, like k_pja_fused.  Those take 1.5 to 1.8 times as long as split launches (a
+// packed bed of 400,000 spheres 412 us a step and 279, of a million 1,435 and 797), so where
+// most spheres get them the launch tells the host, which goes over to the fastest split set if
+// the autotuner had chosen (a bed tuned while it was falling).  A wait is bounded (wait_cycles), latches kFlagTimeout and
 // makes every later wait return at once.
 //
 // All blocks are resident (cooperative launch, one block per SM, no more blocks than the
@@ -740,6 +743,12 @@ __global__ void __launch_bounds__(kFlowThreads, 1) k_flow(const __grid_constant_
     __syncthreads();
   }
   __syncthreads();
+  if (a.flow_told && blockIdx.x == 0 && tid == 0) {  // the host chooses another set when it next steps
+    uint32_t plain = 0;
+    for (uint32_t wave = 0; wave < a.n_waves; ++wave)
+      if (asym || (s_plain[wave >> 5] >> (wave & 31u) & 1u)) plain += a.wave_off[wave + 1] - a.wave_off[wave];
+    if (plain > a.n / 2u) *(volatile uint32_t *)a.flow_told = 1u;
+  }
   for (uint32_t wave = 0; wave < a.n_waves; ++wave)
     if (asym || (s_plain[wave >> 5] >> (wave & 31u) & 1u)) barrier_sweeps(a, iters, G, a.wave_off[wave], a.wave_off[wave + 1]);
 }

@@ -313,3 +313,91 @@ def test_two_simulations_in_two_streams(gg):
     for sim, (x, v) in zip(sims, want):
         assert np.array_equal(sim.pos(), x) and np.array_equal(sim.vel(), v)
         sim.close()
+
+
+def test_lists_that_outgrow_the_chip(gg):
+    """One bed too large for the chip and a small one beside it: the large one's range gets
+    the plain sweeps in the same launch, bit-identical, wrenches too."""
+    big, small = squeezed_column(420000), squeezed_column(20000)
+    for scenes_ in ([big], [small, big, small]):
+        pr = np.concatenate([s.pos_r for s in scenes_])
+        offs = np.concatenate([[0], np.cumsum([s.n for s in scenes_])])
+        out = []
+        for tuning in [7] + flow_sets(gg):
+            sim = gg.Sim(pr, np.zeros((len(pr), 3), np.float32), S.sphere_mass(pr[:, 3]), big.params,
+                         env_offsets=offs, tuning=tuning)
+            for e, s in enumerate(scenes_):
+                sim.set_bodies(s.bodies, e)
+            sim.step(2)
+            out.append([sim.read(f) for f in ("POS", "VEL", "BODY_WRENCH", "CONTACT_IMPULSE")])
+            assert sim.stats()["n_pp"] > 3 * 420000 and sim.stats()["status_flags"] == 0
+            sim.close()
+            assert all(np.array_equal(a, b) for a, b in zip(out[0], out[-1])), tuning
+
+
+def squeezed_column(n):
+    """A column of overlapping spheres, 3.4 contacts each: 3.9 units of cost a sphere, of which
+    the chip takes about 1.26 million."""
+    sc = S.column_collapse(n=n)
+    sc.pos_r[:, :3] *= np.float32(0.88)
+    return sc
+
+
+def test_leaving_a_set_that_no_longer_fits(gg):
+    """Tuned while nothing touches, packed afterwards: the dataflow sweeps report that the
+    bed does not fit, and the simulation goes over to a split set with the same results."""
+    sc = squeezed_column(420000)
+    loose = S.column_collapse(n=420000)
+    sim = gg.Sim.from_scene(loose)
+    sim.step(1)
+    sim.sync()
+    chosen = gg.load().gg_tuning_selected(sim.h)
+    assert "flow" in gg.tuning_flags(chosen)
+    ref = gg.Sim.from_scene(loose, tuning=7)
+    ref.step(1)
+    for s in (sim, ref):
+        s.set_particles(sc.pos_r, sc.vel)
+        for _ in range(3):
+            s.step(1)
+            s.sync()
+    assert "flow" not in gg.tuning_flags(gg.load().gg_tuning_selected(sim.h))
+    for f in ("POS", "VEL", "BODY_WRENCH"):
+        assert np.array_equal(sim.read(f), ref.read(f)), f
+    again = gg.load().gg_tuning_selected(sim.h)
+    sim.step(2)
+    ref.step(2)
+    assert gg.load().gg_tuning_selected(sim.h) == again and np.array_equal(sim.pos(), ref.pos())
+    sim.close()
+    ref.close()
+
+
+def test_free_bodies_with_lists_cut_by_the_capacity(gg):
+    """The plain sweeps with free bodies: their updates between the grid barriers."""
+    sc = pressed_boxes()
+    sc.params = dataclasses.replace(sc.params, max_contacts=2)
+    want, wf = outputs(gg, sc, 7, 3, check=False)
+    assert wf & 1
+    for k in flow_sets(gg):
+        if "half" in gg.tuning_flags(k):
+            continue
+        got, gf = outputs(gg, sc, k, 3, check=False)
+        assert gf == wf
+        for a, b in zip(got, want):
+            assert np.array_equal(a, b), k
+
+
+def test_free_bodies_in_a_small_batch(gg):
+    """Several environments in one range, free bodies in each: the dataflow launch takes them."""
+    a, b = pressed_boxes(), pressed_boxes(2500, v=(0.1, 0.0, -0.1))
+    pr = np.concatenate([a.pos_r, b.pos_r])
+    want = None
+    for tuning in [7] + flow_sets(gg):
+        sim = gg.Sim(pr, np.zeros((len(pr), 3), np.float32), S.sphere_mass(pr[:, 3]), a.params,
+                     env_offsets=[0, a.n, a.n + b.n], tuning=tuning, max_free_bodies=4)
+        for e, s in enumerate((a, b)):
+            sim.set_bodies(s.bodies, e)
+        sim.step(3)
+        got = [sim.read(f) for f in ("POS", "VEL", "BODY_STATE", "BODY_WRENCH")]
+        sim.close()
+        want = want or got
+        assert all(np.array_equal(x, y) for x, y in zip(got, want)), tuning
