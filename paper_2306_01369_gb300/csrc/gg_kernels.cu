@@ -1510,11 +1510,13 @@ __global__ void k_body_state(const DevBody *bodies, uint32_t nbt, float *out) {
 // ---------------------------------------------------------------------------
 
 // Particle count up to which the half-stencil pass takes a thread per row.  Contact stage
-// (both passes) with a thread per particle and per row: 4,096 spheres 26.5 and 21.0 us,
-// 50,000 34.7 and 25.7, a pile of 262,144 60.4 and 55.3; 1,000,000 196 and 202, a batch of
-// 1.8 million 313 and 361 (the chip is full either way, and the extra atomics cost).  The
-// finder's share of pcnt cannot run over its 16 bits: 14 buckets of at most kMaxBucket.
-constexpr uint32_t kSplitRows = 262144;
+// (both passes) with a thread per particle and per row, us: 4,096 spheres 26.5 and 21.0, 50,000
+// 34.7 and 25.7, piles of 262,144 59.0 and 55.3, 400,000 84.0 and 81.9, 524,288 100.4 and 98.3,
+// 700,000 132.7 and 129.1, in no spatial order 600,000 159.8 and 157.7; a batch of 855,000
+// 157.3 and 159.4, a million 196 and 202 (the chip is full either way, and the extra atomics
+// cost).  The finder's share of pcnt cannot run over its 16 bits: 14 buckets of at most
+// kMaxBucket.
+constexpr uint32_t kSplitRows = 700000;
 static_assert(14u * kMaxBucket < 65536u, "a row thread counts its hits in 16 bits");
 
 static inline unsigned grid_for(uint32_t n, int bs) { return (n + bs - 1) / bs > 0 ? (n + bs - 1) / bs : 1; }

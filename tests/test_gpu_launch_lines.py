@@ -143,3 +143,9 @@ def test_traced_images_of_either_form(gg, orc, nb, w, h):
     assert np.array_equal(out[0], orc.render(cam, np.zeros((0, 3)), np.zeros(0), bodies).astype(F32))
     assert np.array_equal(out[2], np.minimum(out[0], out[1]))
     assert (out[1] < out[0]).any() and (out[0] < out[1]).any()
+
+
+@pytest.mark.parametrize("n", [700000, 700001])
+def test_half_stencil_rows_at_the_line(gg, n):
+    """The same on both sides of the count up to which the rows get a thread each."""
+    test_half_stencil_rows(gg, n)
