@@ -70,9 +70,6 @@ constexpr uint32_t kNumHashFactors = sizeof(kHashFactors) / sizeof(kHashFactors[
 constexpr double kCellFactors[] = {2.002, 2.2, 2.5};
 constexpr uint32_t kNumCellFactors = sizeof(kCellFactors) / sizeof(kCellFactors[0]);
 
-// Spheres the dataflow sweeps of a batch take at a time (see gg_flow.cu).
-constexpr uint32_t kWaveParticles = 300000;
-
 constexpr uint32_t kStateMagic = 0x31534747u;  // "GGS1"
 
 struct StateHeader {
@@ -905,9 +902,15 @@ gg_status gg_create_batch(const gg_params *params, uint32_t n_envs, const uint32
       (rc = dalloc(s, &wave_off, (size_t)n_envs + 1)))
     return bail(rc);
   a.tag_step = P.pja_iters + 2u;
+  uint32_t pool = 0;
+  int nsm = 0;
+  const cudaError_t se = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, s->device);
+  if (se != cudaSuccess) return bail(cuda_fail(s, se, "cudaDeviceGetAttribute"));
+  const int per = gg::flow_setup(s->F != 0, &pool);
+  const uint32_t range = per > 0 ? gg::flow_range((uint32_t)(per * nsm), pool) : n;
   std::vector<uint32_t> waves{0u};
   for (uint32_t e2 = 0; e2 < n_envs; ++e2) {
-    if (s->envs[e2].off > waves.back() && s->envs[e2].off + s->envs[e2].n - waves.back() > kWaveParticles)
+    if (s->envs[e2].off > waves.back() && s->envs[e2].off + s->envs[e2].n - waves.back() > range)
       waves.push_back(s->envs[e2].off);
   }
   waves.push_back(n);

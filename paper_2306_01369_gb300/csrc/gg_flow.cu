@@ -54,9 +54,14 @@ namespace {
 constexpr int kFlowThreads = 1024;
 constexpr int kFlowWarps = kFlowThreads / 32;
 constexpr int kEarly = 2;              // records with other blocks' spheres whose estimates a thread asks for ahead
-constexpr uint32_t kTileWeight = 16;   // cost of a 32-sphere tile beside its contacts, in contacts
+// cost of a 32-sphere tile beside its contacts, in contacts (0 and 32 measure the same but for a
+// batch, 420 us of sweeps with 0 and 404 with 16; at 64 a pile of 262,144 no longer fits)
+constexpr uint32_t kTileWeight = 16;
 constexpr uint32_t kBytesPerCost = 24; // ... and no less than its lists and estimates take in shared memory over this
-constexpr uint32_t kMinWork = 640;     // least work worth a block of its own
+// least work worth a block of its own (sweep stage at 1,000, 4,096 and 16,384 spheres: 47, 47 and
+// 49 us, with 320 47, 47 and 47, with 1,280 51, 51 and 51; fewer blocks leave more of the chip
+// to other streams)
+constexpr uint32_t kMinWork = 640;
 constexpr uint32_t kTileMax = 32u * (kMaxK + kMaxKb) + kTileWeight;  // most a tile costs
 constexpr uint32_t kNone = 0xffffffffu;
 constexpr uint32_t kAsymmetric = kFlagPPOverflow | kFlagBucketBound | kFlagListBound | kFlagDebugCheck;
@@ -774,6 +779,15 @@ int flow_setup(bool free, uint32_t *pool) {
   const int per = free ? flow_setup_for<true>(pool) : flow_setup_for<false>(pool);
   if (!per) (void)cudaGetLastError();
   return per;
+}
+
+// A settled bed costs 3.5 to 3.8 a sphere (three contacts, a tile's weight, tiles of uneven
+// lists); with a margin for denser ones that is 302,000 spheres on 152 SMs.  (Sweep stage of
+// a batch of 1.64 million spheres, 2.7 contacts each, with 3.6, 4.2, 6.3 and 8.4: 870, 799, 948
+// and 930 us: too large a range does not fit, too small a one pays the load more often.)
+constexpr double kSettledCost = 4.2;
+uint32_t flow_range(uint32_t grid, uint32_t pool) {
+  return (uint32_t)(grid * (double)((pool - 256u) / kBytesPerCost - kTileMax) / kSettledCost);
 }
 
 // (With all 152 blocks at any size, two simulations in two streams took turns: 4,096 spheres

@@ -61,6 +61,7 @@ constexpr uint32_t kFlowRecords = 10240;      // most record scratch of one bloc
 struct FlowScratch {
   uint32_t blocks, records, bodies;
 };
+uint32_t flow_range(uint32_t grid, uint32_t pool);  // spheres of a settled bed that fit the chip
 uint32_t flow_blocks(uint32_t most);  // blocks that a crowded range of so many spheres can use
 FlowScratch flow_scratch(const StepArgs &a, uint32_t most, uint32_t grid, uint32_t pool);
 int flow_setup(bool free, uint32_t *pool);  // resident blocks per SM, shared memory per block
