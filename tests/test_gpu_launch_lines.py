@@ -149,3 +149,73 @@ def test_traced_images_of_either_form(gg, orc, nb, w, h):
 def test_half_stencil_rows_at_the_line(gg, n):
     """The same on both sides of the count up to which the rows get a thread each."""
     test_half_stencil_rows(gg, n)
+
+
+def test_one_reservation_other_lengths_and_tools(gg):
+    """Reverse passes under one reservation, of other lengths and with another tool: the kept
+    graphs are made anew where they must be, and each pass gives what a simulation of its own
+    gives."""
+    sc = S.diff_scene(n=512, n_steps=6)
+    seed = np.random.default_rng(4).normal(size=(sc.n, 3)).astype(F32)
+    pr = sc.pos_r.copy()      # squeezed, on the container's floor: spheres on each other and on both bodies
+    pr[:, :3] = (pr[:, :3] - pr[:, :3].mean(0)) * np.float32(0.72) + pr[:, :3].mean(0)
+    pr[:, 2] -= (pr[:, 2] - np.float32(0.9) * pr[:, 3]).min()
+
+    def fresh():
+        sim = gg.Sim(pr, None, sc.mass, S.Params(dt=1e-5, mu=0.5, pja_iters=20))
+        sim.set_bodies(sc.bodies)
+        sim.set_trajectory(1, sc.twist[1].astype(F32))
+        sim.tape_reserve(6, 2)
+        return sim
+
+    def run(sim, state, tool, steps):
+        sim.set_state(state)
+        sim.step_taped(tool, steps)
+        return sim.backward(seed)
+
+    kept = fresh()
+    state = kept.state()
+    for tool, steps in ((1, 4), (1, 6), (1, 6), (0, 6), (0, 3), (1, 3), (1, 4)):
+        got = run(kept, state, tool, steps)
+        one = fresh()
+        want = run(one, state, tool, steps)
+        one.close()
+        assert np.array_equal(got[0], want[0]) and got[1] == want[1], (tool, steps)
+        assert np.abs(got[0]).max() > 0
+    kept.close()
+
+
+@pytest.mark.parametrize("n", [4000, 20000, 70000])
+def test_reverse_pass_lanes_against_eight(gg, n):
+    """8, 4 and 2 lanes a particle (by the particle count) on the same contacts: a squeezed bed
+    of 512 spheres with the scoop, filled up with spheres that touch nothing, against the bed
+    alone, whose 8-lane gradients the oracle's tests pin.  Same terms, summed in another order:
+    at most 512 particles x 20 sweeps of float32 sums with carried errors, 1e-4 of the largest
+    component of each kind (forces, torques, mu)."""
+    sc = S.diff_scene(n=512, n_steps=4)
+    rng = np.random.default_rng(9)
+    pr = sc.pos_r[:512].copy()
+    pr[:, :3] = (pr[:, :3] - pr[:, :3].mean(0)) * np.float32(0.6) + pr[:, :3].mean(0)
+    k = np.arange(n - 512)
+    fill = np.empty((n - 512, 4), F32)
+    fill[:, :3] = 0.005 * np.stack([k % 4 - 1.5, k // 4 % 4 - 1.5, k // 16 + 200], -1)   # a tower over the container
+    fill[:, 3] = 0.002
+    seed = rng.normal(size=(512, 3)).astype(F32)
+    out = []
+    for extra in (0, n - 512):
+        x = np.concatenate([pr, fill[:extra]])
+        sim = gg.Sim(x, None, S.sphere_mass(x[:, 3]), S.Params(dt=1e-5, mu=0.5, pja_iters=20, max_contacts=24))
+        sim.set_bodies(sc.bodies)
+        sim.set_trajectory(1, sc.twist[1].astype(F32))
+        sim.tape_reserve(3, 3)
+        sim.step_taped(1, 3)
+        counts = np.diff(sim.contacts()["pp_off"].astype(np.int64))
+        assert counts[:512].max() > 8 and not counts[512:].any()
+        tw, mu = sim.backward(np.concatenate([seed, np.zeros((extra, 3), F32)]))
+        sim.close()
+        out.append((np.asarray(tw, np.float64), float(mu)))
+    (a, ma), (b, mb) = out
+    for k in (slice(0, 3), slice(3, 6)):
+        assert np.abs(a[:, k]).max() > 0
+        assert np.abs(a[:, k] - b[:, k]).max() <= 1e-4 * np.abs(a[:, k]).max()
+    assert ma != 0 and abs(ma - mb) <= 1e-4 * abs(ma)

@@ -824,3 +824,15 @@ def test_step_io_equals_the_three_calls(gg, torch, pinned):
     a.step_io(pos_h, vel_h, other)
     b.step(1)
     assert np.array_equal(other.numpy()[:4 * sc.n].reshape(-1, 4), b.pos())
+
+
+@pytest.mark.parametrize("tuning", [23, 24, 25])
+def test_column_collapse_full_size_dataflow_sets_at_8n(gg, orc, column_800, tuning):
+    """The sets whose sweeps run in one launch, the benchmark's configuration among them, at
+    full size (see _column_check)."""
+    _column_check(gg, orc, column_800, tuning, 8)
+
+
+def test_every_launch_shape_has_its_full_size_check(gg):
+    """The two full-size tests name the sets 1-25: a set added later has to join them."""
+    assert gg.load().gg_tuning_count() == 25
