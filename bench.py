@@ -251,6 +251,12 @@ def stage_kernels(flags):
     return sweep, contacts
 
 
+def running_flags(flags, kernels_per_step, iters):
+    """`flags` without "flow" where the step runs the split launches all the same (more free
+    bodies than those sweeps take, for instance): a launch per sweep shows in the count."""
+    return flags - {"flow"} if kernels_per_step > iters else flags
+
+
 def profile_traffic(kernel: str, workload: str, kernel_digest: str):
     """ncu DRAM bytes per launch of `kernel` (the contact stage's kernels summed) from its
     committed profile summary ("key: value" lines) on this workload, if it was taken on
@@ -766,13 +772,14 @@ def measure(sim, sc, steps, stream, torch, flush, workload="column", readback=No
         avg_s = total_ms * 1e-3 / launches
         per_launch = total_bytes / launches
         achieved = per_launch / avg_s / 1e9
-        return {"bound": "hbm", "kernel": kernel, "achieved": achieved, "peak": peak, "unit": "GB/s",
+        return {"bound": "latency" if kernel == "k_flow" else "hbm", "kernel": kernel, "achieved": achieved, "peak": peak, "unit": "GB/s",
                 "frac": achieved / peak, "peak_kind": f"{peak_kind} hbm_gbs (copy), burst",
                 "traffic": profile_traffic(kernel, workload, digest), "bytes_per_launch": per_launch,
                 "avg_launch_us": avg_s * 1e6, "share_of_step": total_ms / sampled_ms,
                 "sampled_steps": len(sampled)}
 
-    sweep_kernel, contact_kernels = stage_kernels(sim.tuning_flags)
+    sweep_kernel, contact_kernels = stage_kernels(
+        running_flags(sim.tuning_flags, sim.kernels_per_step, sc.params.pja_iters))
     if sweep_kernel == contact_kernels:   # detection and sweeps in one launch per step
         roofs = [roof(sweep_kernel, pja_ms + con_ms, pja_b + con_b, len(sampled)), None]
     else:

@@ -58,3 +58,8 @@ def test_committed_profiles_are_readable_and_name_their_command():
             assert workload is not None, path
             assert bench.profile_traffic(kernel, workload, kv["kernel_digest"].strip()) == \
                 float(kv["dram_bytes_per_launch"])
+
+
+def test_split_launches_of_a_dataflow_set_are_named():
+    assert bench.stage_kernels(bench.running_flags({"flow", "lists", "half"}, 8, 20))[0] == "k_flow"
+    assert bench.stage_kernels(bench.running_flags({"flow", "lists", "half"}, 48, 20))[0] == "k_pja"
