@@ -419,7 +419,7 @@ GG_API uint32_t gg_tuning_selected(const gg_sim *sim);
  * Every set gives the same results; the bits only describe how the step is launched. */
 #define GG_TUNE_LISTS 1u /* binning by per-bucket linked lists (else the counting sort) */
 #define GG_TUNE_FUSED 2u /* all sweeps in one cooperative launch with grid barriers */
-#define GG_TUNE_LEAN 4u  /* the sweep capped at 40 registers */
+#define GG_TUNE_LEAN 4u  /* the sweep capped at 56 registers */
 #define GG_TUNE_HALF 8u  /* pair search over half the stencil, then a mirroring pass */
 #define GG_TUNE_DETECT 16u /* detection and all sweeps in one cooperative launch, a grid barrier
                               between them (the paper's TwoLoopsFused, Sec. II-D); without free
@@ -432,8 +432,9 @@ GG_API uint32_t gg_tuning_selected(const gg_sim *sim);
                                 and computes the responses there, not from stored records */
 #define GG_TUNE_FLOW 256u    /* all sweeps in one launch ordered by data: the contact records stay in
                                 shared memory, partners exchange tagged velocity estimates, no
-                                barrier (with more than 8 free bodies, free bodies in a batch, or pja_weight = 1 the
-                                set runs the split launches) */
+                                barrier (with more than 8 free bodies, free bodies in a batch of more
+                                spheres than one range takes, about 300,000, or pja_weight = 1 the set
+                                runs the split launches) */
 
 GG_API uint32_t gg_tuning_flags(uint32_t k);
 

@@ -53,7 +53,7 @@ const gg::LaunchShape kShapes[] = {
     shape(256, 0),  shape(128, 0), shape(512, 0), shape(64, 0),       // 1-4: sort, per-launch sweeps
     shape(256, 0, 1024), shape(256, 0, 512),                           // 5-6: all sweeps in one launch
     shape(256, kL), shape(128, kL),                                    // 7-8: lists
-    shape(256, kL | kLean), shape(256, kLean),                         // 9-10: 40-register sweeps
+    shape(256, kL | kLean), shape(256, kLean),                         // 9-10: 56-register sweeps
     shape(256, kL | kHalf), shape(256, kL | kLean | kHalf), shape(256, kHalf),  // 11-13: half stencil
     shape(256, kDet), shape(256, kL | kDet),                           // 14-15: TwoLoopsFused
     shape(128, kSerp | kPre), shape(128, kL | kSerp | kPre), shape(128, kL | kHalf | kSerp | kPre),  // 16-18

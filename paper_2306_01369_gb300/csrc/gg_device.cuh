@@ -175,7 +175,8 @@ struct StepArgs {
   uint32_t *ccount; // pp | body << 8
   uint32_t *cj;     // [K][n] partner id
   float4 *cn;       // [K][n] normal (partner -> particle), psi
-  float4 *clam;     // [K][n] accumulated impulse, partner id in w (the sweeps read it there)
+  float4 *clam;     // [K][n] accumulated impulse; while sweeps run from it, the partner id in w (the dataflow
+                    // sweeps keep impulses and ids on chip and leave 0 there)
   uint32_t *bj;     // [Kb][n] global body index
   float4 *bn;       // [Kb][n] normal (body -> particle), psi
   float4 *bxc;      // [Kb][n] contact point

@@ -4,8 +4,8 @@
 // What bounds a sweep as a launch of its own: 4.2 us at 4,096 spheres and 5.0 at 262,144
 // with a fifth of them in contact, whatever the bytes -- a launch (0.9 us) and a chain of
 // four dependent loads (counts, partner ids, partners' estimates, bodies) -- and, where
-// every sphere is in contact, the re-reading of the records (44 bytes per contact and
-// sweep).  Here a block loads the contact records of its spheres once, keeps them in
+// every sphere is in contact, the re-reading of the records (48 bytes per contact and
+// sweep: normal, impulse in and out).  Here a block loads the contact records of its spheres once, keeps them in
 // shared memory for all I sweeps, impulses included, and what a sweep moves through L2 is
 // 16 bytes out per sphere that other blocks' spheres touch and 16 bytes in per such contact.
 // Measured (sweep stage of a step, 20 iterations, us): 4,096 spheres 84 -> 48, 16,384
@@ -187,7 +187,7 @@ __device__ __forceinline__ void barrier_sweeps(const StepArgs &a, uint32_t iters
       const uint32_t cc = a.ccount[i];
       if (!(cc & 0xffffu)) {  // (left out by the contact build, but a cut list elsewhere may name it)
         const float4 b = base_velocity(a, a.vel_id[i]);
-        a.U[0][i] = make_float4(b.x, b.y, b.z, a.lit ? b.w : 0.f);
+        a.U[0][i] = make_float4(b.x, b.y, b.z, 0.f);
       }
       for (uint32_t c = 0; c < (cc & 0xffu); ++c) a.clam[(size_t)c * n + i] = no_impulse(a.cj[(size_t)c * n + i]);
       for (uint32_t c = 0; c < 3 * ((cc >> 8) & 0xffu); ++c) a.blam[(size_t)(c % 3) * KbN + (size_t)(c / 3) * n + i] = 0.f;
@@ -298,7 +298,7 @@ __device__ __forceinline__ uint32_t place_of(const Block &k, uint32_t j, uint32_
 }
 
 struct Sweep {
-  uint32_t s, iters;        // iteration, iterations
+  uint32_t s;               // iteration
   uint32_t tag, pub;        // tag of U^s, tag under which U^{s+1} is published
 };
 
@@ -371,7 +371,6 @@ __device__ __forceinline__ void sweeps(const StepArgs &a, const Block &k, uint32
                                        uint32_t tag0, uint32_t out0, Waits &wt) {
   const uint32_t tid = threadIdx.x;
   Sweep w;
-  w.iters = iters;
   for (uint32_t s = 0; s < iters; ++s) {
     w.s = s;
     w.tag = tag0 + s;
