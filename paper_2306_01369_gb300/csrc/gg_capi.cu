@@ -335,7 +335,7 @@ void flow_release(gg_sim *s) {
 // The scratch of the dataflow sweeps, held while a set that runs them is selected or still to
 // be tried (released by an autotuning that chose another): two tagged estimates a sphere, and per block that can get work the records that may
 // not fit on chip and the contacts with bodies.  (152 blocks of the largest size, 87 MB, were
-// held by every simulation; now 1,000 spheres hold 1 MB and 4,096 hold 5.)  Nothing to do
+// held by every simulation; now 1,000 spheres hold less than 1 MB and 4,096 hold 4.)  Nothing to do
 // where the sweeps cannot run.
 gg_status flow_reserve(gg_sim *s, cudaStream_t st) {
   StepArgs &a = s->a;
