@@ -271,7 +271,7 @@ def test_memory_of_small_simulations(gg):
     """A simulation whose set never runs the dataflow sweeps holds none of their scratch, and
     a small one little (152 blocks' worth would be 87 MB): 32 bytes a sphere, and at 4,096
     spheres 16 bytes for each of 131 blocks' at most 1,279 + 656 contacts with bodies, a few
-    MB, with the driver's 2 MB granularity for each of the seven buffers."""
+    MB, with cudaMalloc's 2 MB granularity for each of the seven buffers."""
     torch = need_gpu()
     sc = squeezed(4096)
 
